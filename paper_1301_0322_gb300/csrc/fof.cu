@@ -187,15 +187,18 @@ extern "C" int cola_fof(cola_plan* plan, const float* s, int32_t b_num, int32_t 
   for (int k = 0; k < nthr; ++k) thr.v[k] = thresholds[k];
   cudaStream_t st = (cudaStream_t)stream;
   Workspace& w = plan->ws;
-  // scratch: cell bins in the force-mesh region, union-find arrays in the half spectra
+  // scratch: cell bins in the force-mesh region, union-find arrays in the half spectra.  With
+  // cells of one mesh cell (nbins = ng^3) four bin arrays do not fit in the 3 ng^3 floats, so the
+  // counts, dead once the scan is done, share the buffer of the group sizes, which are written
+  // after it (a half spectrum holds more than ng^3 floats).
   Tiles cells{};
   cells.nbins = nc * nc * nc;
-  int* counts = reinterpret_cast<int*>(w.freal);
-  int* offsets = counts + cells.nbins;
+  int* offsets = reinterpret_cast<int*>(w.freal);
   int* cursor = offsets + cells.nbins + 1;
   int* scan_blocks = cursor + cells.nbins;
   int* parent = reinterpret_cast<int*>(w.meshA);
   int* gsize = reinterpret_cast<int*>(w.meshG[1]);
+  int* counts = gsize;
   int* minp = reinterpret_cast<int*>(w.meshG[2]);
   const int64_t n = g.np3;
   COLA_CUDA_CHECK(cudaMemsetAsync(counts, 0, sizeof(int) * cells.nbins, st));

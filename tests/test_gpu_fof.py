@@ -85,3 +85,22 @@ def test_union_retry_limit_reports_timeout_and_recovers(cola):
         cola.cola_set_fof_union_tries(plan.handle, -1)
     cola.cola_set_fof_union_tries(plan.handle, 1 << 20)
     assert check(cola, plan, s32, n_p, ng, box) >= 1
+
+
+@pytest.mark.parametrize("n_p,ng", [(32, 64), (32, 96), (32, 32)])
+def test_fof_stays_inside_its_workspace(cola, n_p, ng):
+    # linking cells of one mesh cell need the most scratch: nothing behind the workspace may change
+    from paper_1301_0322_gb300 import cola as binding
+    cfg = binding._make_config(n_p, ng, 50.0)
+    h = binding.cola_plan_create(cfg)
+    nbytes = binding.cola_workspace_bytes(h)
+    buf = torch.full((nbytes + (1 << 20),), 0x5A, dtype=torch.uint8, device="cuda")
+    assert buf.data_ptr() % 256 == 0
+    binding.cola_set_workspace(h, buf[:nbytes])
+    s = torch.from_numpy(inputs.clustered_displacements(n_p, 50.0, 3)).cuda()
+    group = torch.empty(n_p**3, dtype=torch.int32, device="cuda")
+    size = torch.empty_like(group)
+    binding.cola_fof(h, s, 1, 5, 25, group, size, None, None)
+    binding.cola_status(h)
+    assert bool((buf[nbytes:] == 0x5A).all())
+    binding.cola_plan_destroy(h)
