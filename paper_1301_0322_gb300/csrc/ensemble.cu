@@ -179,12 +179,15 @@ __global__ void __launch_bounds__(NT, 512 / NT) ke_deposit(const BoxDesc* __rest
 
 // column passes: kind 0 = forward y, 1 = z with the Green's function, 2 = inverse y (three
 // outputs); single-buffer strips of W = NT / T(N) columns, stage twiddles from shared memory
-// (the bodies of the single-box passes at 128-256; the z pass keeps phi in A)
+// (the bodies of the single-box passes, one column per thread)
 template <int NT, int KIND, int V>
 __global__ void __launch_bounds__(NT, 512 / NT) ke_cols(const BoxDesc* __restrict__ boxes, const int* __restrict__ starts,
                                               int nbox) {
   extern __shared__ __align__(16) unsigned long long ens_smem[];
   float2* sm = reinterpret_cast<float2*>(ens_smem);
+  __shared__ uint32_t slot;
+  // the longest transforms hold 24 elements a thread
+  const std::conditional_t<KIND == 0, NoPark, Park<NT, 24, float2>> park(&slot);
   const int total = __ldg(starts + nbox);
   BoxCursor cur(starts, nbox, blockIdx.x);
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
@@ -197,15 +200,14 @@ __global__ void __launch_bounds__(NT, 512 / NT) ke_cols(const BoxDesc* __restric
     using C = FFTConfV<N, V>;                                                                             \
     constexpr int W = NT / C::T, nbx = (N / 2 + 1 + W - 1) / W;                                           \
     const int bx = local % nbx, slab = local / nbx;                                                       \
-    if (KIND == 0) {                                                                                      \
+    if constexpr (KIND == 0) {                                                                            \
       float2* stab = sm + N * W;                                                                          \
       stw_fill<C, 1>(stab, d.tw, threadIdx.x, NT);                                                        \
-      cols_body<N, W, false, C>(d.A, (int64_t)N * d.P, d.P, N / 2 + 1, SmemTw<C>{stab}, bx, slab, sm);    \
-    } else if (KIND == 1) {                                                                               \
-      z_green_wide_body<N, W, 0, C>(d.A, d.Gz, nullptr, nullptr, d.kf, d.deconv, d.norm, d.tw, d.err, bx, \
-                                    slab, sm);                                                            \
+      cols_body<N, W, 1, false, float2, C>(d.A, (int64_t)N * d.P, d.P, N / 2 + 1, SmemTw<C>{stab}, bx, slab, sm);    \
+    } else if constexpr (KIND == 1) {                                                                     \
+      z_green_body<N, W, 1, float2, C>(d.A, d.Gz, d.kf, d.deconv, d.norm, d.tw, bx, slab, sm, park);      \
     } else {                                                                                              \
-      y_inv3_wide_body<N, W, C>(d.A, d.Gy, d.Gz, d.kf, d.tw, bx, slab, sm);                               \
+      y_inv3_body<N, W, 1, float2, C>(d.A, d.Gy, d.Gz, d.kf, d.tw, bx, slab, sm, park);                   \
     }                                                                                                     \
   } break;
       COLA_ENS_SIZES(X)
@@ -215,6 +217,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) ke_cols(const BoxDesc* __restric
     }
     __syncthreads();
   }
+  park.close();
 }
 
 // Stage twiddle tables (fft.cuh) of the inverse-x transforms of every ensemble size, behind the

@@ -26,10 +26,84 @@ __device__ __forceinline__ float2 c_mul(float2 a, float2 b) {
 }
 __device__ __forceinline__ float2 c_conj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 c_scale(float2 a, float s) { return make_float2(__fmul_rn(a.x, s), __fmul_rn(a.y, s)); }
-// multiply by -i (forward sign) or +i (inverse sign)
+// a + r b and a - r b with r = -i (forward sign) or +i (inverse sign)
 template <bool INV>
-__device__ __forceinline__ float2 c_rot(float2 a) {
-  return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+__device__ __forceinline__ float2 c_add_rot(float2 a, float2 b) {
+  return INV ? make_float2(__fsub_rn(a.x, b.y), __fadd_rn(a.y, b.x)) : make_float2(__fadd_rn(a.x, b.y), __fsub_rn(a.y, b.x));
+}
+template <bool INV>
+__device__ __forceinline__ float2 c_sub_rot(float2 a, float2 b) {
+  return c_add_rot<!INV>(a, b);
+}
+__device__ __forceinline__ float2 c_fma(float s, float2 a, float2 b) { return make_float2(fmaf(s, a.x, b.x), fmaf(s, a.y, b.y)); }
+// a + i s b
+__device__ __forceinline__ float2 c_fma_i(float s, float2 b, float2 a) { return make_float2(fmaf(-s, b.y, a.x), fmaf(s, b.x, a.y)); }
+
+// Two complex values at once, as the pair of their real parts and the pair of their imaginary
+// parts: the arithmetic of a transform over two columns then runs in packed float32
+// instructions (add, mul, fma .f32x2), each of which rounds its two lanes as the scalar one
+// does, so both columns get the bits of the scalar transform for half of its instructions
+// (twiddles, addresses and exchange accesses are shared as well).
+struct alignas(16) cpair {
+  float2 re, im;
+};
+__device__ __forceinline__ unsigned long long p_bits(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 p_value(unsigned long long v) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(v));
+  return d;
+}
+__device__ __forceinline__ float2 p_add(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(p_bits(a)), "l"(p_bits(b)));
+  return p_value(r);
+}
+__device__ __forceinline__ float2 p_sub(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(p_bits(a)), "l"(p_bits(b)));
+  return p_value(r);
+}
+__device__ __forceinline__ float2 p_mul(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(p_bits(a)), "l"(p_bits(b)));
+  return p_value(r);
+}
+__device__ __forceinline__ float2 p_fma(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(p_bits(a)), "l"(p_bits(b)), "l"(p_bits(c)));
+  return p_value(r);
+}
+// A product that may feed an add, as two scalar instructions (the same time in the float32 pipe):
+// the compiler fuses a packed product into a following packed add, .rn or not, which would round
+// once where the scalar code rounds twice.
+__device__ __forceinline__ float2 p_mul_rn(float2 a, float2 b) { return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)); }
+__device__ __forceinline__ float2 p_dup(float s) { return make_float2(s, s); }
+__device__ __forceinline__ cpair c_add(cpair a, cpair b) { return {p_add(a.re, b.re), p_add(a.im, b.im)}; }
+__device__ __forceinline__ cpair c_sub(cpair a, cpair b) { return {p_sub(a.re, b.re), p_sub(a.im, b.im)}; }
+// both lanes by the same factor w (rounded as c_mul(float2, float2))
+__device__ __forceinline__ cpair c_mul(cpair a, float2 w) {
+  const float2 wr = p_dup(w.x), wi = p_dup(w.y), nwi = p_dup(-w.y);
+  return {p_fma(a.re, wr, p_mul(a.im, nwi)), p_fma(a.re, wi, p_mul(a.im, wr))};
+}
+// lane by lane: a.lane0 * s.x, a.lane1 * s.y
+__device__ __forceinline__ cpair c_scale(cpair a, float2 s) { return {p_mul_rn(a.re, s), p_mul_rn(a.im, s)}; }
+template <bool INV>
+__device__ __forceinline__ cpair c_add_rot(cpair a, cpair b) {
+  return INV ? cpair{p_sub(a.re, b.im), p_add(a.im, b.re)} : cpair{p_add(a.re, b.im), p_sub(a.im, b.re)};
+}
+template <bool INV>
+__device__ __forceinline__ cpair c_sub_rot(cpair a, cpair b) {
+  return c_add_rot<!INV>(a, b);
+}
+__device__ __forceinline__ cpair c_fma(float s, cpair a, cpair b) {
+  return {p_fma(p_dup(s), a.re, b.re), p_fma(p_dup(s), a.im, b.im)};
+}
+__device__ __forceinline__ cpair c_fma_i(float s, cpair b, cpair a) {
+  return {p_fma(p_dup(-s), b.im, a.re), p_fma(p_dup(s), b.re, a.im)};
 }
 
 // Compile-time sine/cosine (Taylor series in double; arguments in [0, 2 pi)) for the constant
@@ -58,26 +132,25 @@ struct ConstTw {
   static constexpr float im = (INV ? 1.0f : -1.0f) * (float)cx_sin(2.0 * kPi * K / R);
 };
 
-// y <- x * exp(-+2 pi i K / R), with the trivial angles special-cased
-template <int R, int K, bool INV>
-__device__ __forceinline__ float2 mul_const_tw(float2 x) {
+// x * exp(-+2 pi i K / R) (a quarter turn is left to c_add_rot / c_sub_rot)
+template <int R, int K, bool INV, class V>
+__device__ __forceinline__ V mul_const_tw(V x) {
   if constexpr (K == 0) {
     return x;
-  } else if constexpr (4 * K == R) {
-    return c_rot<INV>(x);
   } else {
     return c_mul(x, make_float2(ConstTw<R, K, INV>::re, ConstTw<R, K, INV>::im));
   }
 }
 
-// ---- small in-register DFTs -------------------------------------------------------------
+// ---- small in-register DFTs (V: float2, one value, or cpair, two at once) -----------------
 template <int R, bool INV>
 struct DFT;
 
 template <bool INV>
 struct DFT<2, INV> {
-  __device__ __forceinline__ static void run(float2* v) {
-    const float2 a = v[0], b = v[1];
+  template <class V>
+  __device__ __forceinline__ static void run(V* v) {
+    const V a = v[0], b = v[1];
     v[0] = c_add(a, b);
     v[1] = c_sub(a, b);
   }
@@ -85,27 +158,29 @@ struct DFT<2, INV> {
 
 template <bool INV>
 struct DFT<3, INV> {
-  __device__ __forceinline__ static void run(float2* v) {
+  template <class V>
+  __device__ __forceinline__ static void run(V* v) {
     // omega = exp(-+2 pi i / 3) = -1/2 + i s,  s = -+sqrt(3)/2
     constexpr float s = INV ? 0.866025403784438647f : -0.866025403784438647f;
-    const float2 t1 = c_add(v[1], v[2]);
-    const float2 t2 = make_float2(fmaf(-0.5f, t1.x, v[0].x), fmaf(-0.5f, t1.y, v[0].y));
-    const float2 t3 = c_sub(v[1], v[2]);
+    const V t1 = c_add(v[1], v[2]);
+    const V t2 = c_fma(-0.5f, t1, v[0]);
+    const V t3 = c_sub(v[1], v[2]);
     v[0] = c_add(v[0], t1);
-    v[1] = make_float2(fmaf(-s, t3.y, t2.x), fmaf(s, t3.x, t2.y));
-    v[2] = make_float2(fmaf(s, t3.y, t2.x), fmaf(-s, t3.x, t2.y));
+    v[1] = c_fma_i(s, t3, t2);
+    v[2] = c_fma_i(-s, t3, t2);
   }
 };
 
 template <bool INV>
 struct DFT<4, INV> {
-  __device__ __forceinline__ static void run(float2* v) {
-    const float2 t0 = c_add(v[0], v[2]), t1 = c_sub(v[0], v[2]);
-    const float2 t2 = c_add(v[1], v[3]), t3 = c_rot<INV>(c_sub(v[1], v[3]));
+  template <class V>
+  __device__ __forceinline__ static void run(V* v) {
+    const V t0 = c_add(v[0], v[2]), t1 = c_sub(v[0], v[2]);
+    const V t2 = c_add(v[1], v[3]), t3 = c_sub(v[1], v[3]);
     v[0] = c_add(t0, t2);
     v[2] = c_sub(t0, t2);
-    v[1] = c_add(t1, t3);
-    v[3] = c_sub(t1, t3);
+    v[1] = c_add_rot<INV>(t1, t3);
+    v[3] = c_sub_rot<INV>(t1, t3);
   }
 };
 
@@ -114,13 +189,24 @@ template <int R, bool INV>
 struct DFT {
   static_assert(R % 2 == 0 && R <= 16, "unsupported radix");
   static constexpr int H = R / 2;
-  template <int... K>
-  __device__ __forceinline__ static void combine(float2* v, const float2* e, const float2* o,
-                                                 std::integer_sequence<int, K...>) {
-    ((v[K] = c_add(e[K], mul_const_tw<R, K, INV>(o[K])), v[K + H] = c_sub(e[K], mul_const_tw<R, K, INV>(o[K]))), ...);
+  template <int K, class V>
+  __device__ __forceinline__ static void combine_one(V* v, const V& e, const V& o) {
+    if constexpr (4 * K == R) {
+      v[K] = c_add_rot<INV>(e, o);
+      v[K + H] = c_sub_rot<INV>(e, o);
+    } else {
+      const V p = mul_const_tw<R, K, INV>(o);
+      v[K] = c_add(e, p);
+      v[K + H] = c_sub(e, p);
+    }
   }
-  __device__ __forceinline__ static void run(float2* v) {
-    float2 e[H], o[H];
+  template <class V, int... K>
+  __device__ __forceinline__ static void combine(V* v, const V* e, const V* o, std::integer_sequence<int, K...>) {
+    (combine_one<K>(v, e[K], o[K]), ...);
+  }
+  template <class V>
+  __device__ __forceinline__ static void run(V* v) {
+    V e[H], o[H];
 #pragma unroll
     for (int i = 0; i < H; ++i) {
       e[i] = v[2 * i];
@@ -199,6 +285,12 @@ __device__ __forceinline__ int xpad(int n) {
   constexpr int shift = R0 >= 16 ? 4 : 3;
   return n + (n >> shift);
 }
+template <int R0, int... Rs>
+__host__ __device__ constexpr int last_radix_of(Radices<R0, Rs...>) {
+  int last = R0;
+  for (int r : {R0, Rs...}) last = r;
+  return last;
+}
 template <class C>
 __host__ __device__ constexpr int first_radix() {
   return FirstRadix<typename C::radices>::value;
@@ -267,8 +359,8 @@ __device__ __forceinline__ void stw_fill(float2* dst, const float2* __restrict__
 template <class C, bool TIGHT = false>
 struct SmemTw {
   const float2* base;
-  template <int R, int NS, bool INV>
-  __device__ __forceinline__ void apply(unsigned j, float2* x) const {
+  template <int R, int NS, bool INV, class V>
+  __device__ __forceinline__ void apply(unsigned j, V* x) const {
     constexpr int off = stw_offset_of(typename C::radices{}, NS, TIGHT), p = stw_pitch(R, TIGHT);
     const float4* q = reinterpret_cast<const float4*>(base + off + j * p);
 #pragma unroll
@@ -299,8 +391,8 @@ struct Stockham {
   // twiddle and in-register DFT of every butterfly this thread owns (butterfly j = t + T q,
   // inputs v[q R + r] = x[j + r N/R]), for a stage of radix R after NS points were combined
   // (tw: the base table, or an SmemTw stage table)
-  template <int R, int NS, class TW>
-  __device__ __forceinline__ static void compute(float2 (&v)[E], int t, const TW& tw) {
+  template <int R, int NS, class V, class TW>
+  __device__ __forceinline__ static void compute(V (&v)[E], int t, const TW& tw) {
 #pragma unroll
     for (int q = 0; q < E / R; ++q) {
       if constexpr (NS > 1) {
@@ -335,13 +427,13 @@ struct Stockham {
   }
 
   // Run the stages NS.. of the radix list.  v holds the inputs of the first listed stage.
-  // mem(n) -> float2& : exchange buffer slot for element n of this thread's sequence.
+  // mem(n) -> V& : exchange buffer slot for element n of this thread's sequence.
   // store(n, x)       : final output of element n.
   // before() / after(): called by every thread just before / after the first block barrier,
   // the one that separates the first stage's reads of its inputs from the first exchange
   // writes (a block that reads its inputs from a buffer may hand the buffer on after it).
-  template <int NS, int R, int... Rest, class TW, class Mem, class Store, class Before, class After>
-  __device__ __forceinline__ static void run(float2 (&v)[E], int t, const TW& tw, Mem& mem, Store& store,
+  template <int NS, int R, int... Rest, class V, class TW, class Mem, class Store, class Before, class After>
+  __device__ __forceinline__ static void run(V (&v)[E], int t, const TW& tw, Mem& mem, Store& store,
                                              Before& before, After& after) {
     compute<R, NS>(v, t, tw);
     if constexpr (sizeof...(Rest) == 0) {
@@ -371,8 +463,34 @@ struct Stockham {
     }
   }
 
-  template <int... Rs, class TW, class Mem, class Store, class Before, class After>
-  __device__ __forceinline__ static void run_all(Radices<Rs...>, float2 (&v)[E], int t, const TW& tw, Mem& mem,
+  // The stages NS.. with the result left in registers, in the last stage's order.
+  template <int NS, int R, int... Rest, class V, class TW, class Mem>
+  __device__ __forceinline__ static void run_regs(V (&v)[E], int t, const TW& tw, Mem& mem) {
+    compute<R, NS>(v, t, tw);
+    if constexpr (sizeof...(Rest) > 0) {
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < E / R; ++q)
+#pragma unroll
+        for (int r = 0; r < R; ++r) mem(out_index<R, NS>(t, q, r)) = v[q * R + r];
+      __syncthreads();
+      constexpr int R2 = FirstRadix<Radices<Rest...>>::value;
+#pragma unroll
+      for (int q = 0; q < E / R2; ++q)
+#pragma unroll
+        for (int r = 0; r < R2; ++r) v[q * R2 + r] = mem(t + T * q + r * (N / R2));
+      run_regs<NS * R, Rest...>(v, t, tw, mem);
+    } else {
+      static_assert(NS * R == N, "radix list does not multiply to N");
+    }
+  }
+  template <int... Rs, class V, class TW, class Mem>
+  __device__ __forceinline__ static void run_regs_all(Radices<Rs...>, V (&v)[E], int t, const TW& tw, Mem& mem) {
+    run_regs<1, Rs...>(v, t, tw, mem);
+  }
+
+  template <int... Rs, class V, class TW, class Mem, class Store, class Before, class After>
+  __device__ __forceinline__ static void run_all(Radices<Rs...>, V (&v)[E], int t, const TW& tw, Mem& mem,
                                                  Store& store, Before& before, After& after) {
     run<1, Rs...>(v, t, tw, mem, store, before, after);
   }
@@ -387,7 +505,7 @@ __device__ __forceinline__ void fft_1d_hooked(int t, const TW& tw, Load& load, M
   static_assert(C::N == N, "configuration of another length");
   constexpr int E = C::E, T = C::T;
   constexpr int R0 = FirstRadix<typename C::radices>::value;
-  float2 v[E];
+  decltype(load(0)) v[E];  // float2 or cpair
 #pragma unroll
   for (int q = 0; q < E / R0; ++q)
 #pragma unroll
@@ -399,6 +517,27 @@ template <int N, int TWS, bool INV, class C = FFTConf<N>, class TW, class Load, 
 __device__ __forceinline__ void fft_1d(int t, const TW& tw, Load& load, Mem& mem, Store& store) {
   auto none = [] {};
   fft_1d_hooked<N, TWS, INV, C>(t, tw, load, mem, store, none, none);
+}
+
+// Transform of values in registers: u[m] is element n = t + T m (0 <= m < E) before and after.
+// Both the first stage's inputs and the last stage's outputs of a thread are the elements
+// congruent to t modulo T, so a thread can go from one transform to the next without an exchange.
+// (The first exchange starts with a block barrier; none follows the last one's reads.)
+template <int N, int TWS, bool INV, class C = FFTConf<N>, class V, class TW, class Mem>
+__device__ __forceinline__ void fft_regs(V (&u)[C::E], int t, const TW& tw, Mem& mem) {
+  static_assert(C::N == N, "configuration of another length");
+  constexpr int E = C::E;
+  constexpr int R0 = FirstRadix<typename C::radices>::value, RL = last_radix_of(typename C::radices{});
+  V v[E];
+#pragma unroll
+  for (int q = 0; q < E / R0; ++q)
+#pragma unroll
+    for (int r = 0; r < R0; ++r) v[q * R0 + r] = u[q + r * (E / R0)];
+  Stockham<N, E, TWS, INV>::run_regs_all(typename C::radices{}, v, t, tw, mem);
+#pragma unroll
+  for (int q = 0; q < E / RL; ++q)
+#pragma unroll
+    for (int r = 0; r < RL; ++r) u[q + r * (E / RL)] = v[q * RL + r];
 }
 
 }  // namespace cola

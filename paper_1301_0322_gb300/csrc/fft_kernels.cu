@@ -15,40 +15,18 @@ __host__ __device__ constexpr int x_rows() {
   return FFTConf<N / 2>::T >= 256 ? 1 : 256 / FFTConf<N / 2>::T;
 }
 
-// Columns per block of the stand-alone column passes: 8 (64-byte row segments) for the 16-element
-// transforms of length 1024 and 2048, whose one exchange buffer leaves room for them (the
-// two-buffer force passes at those lengths use col_width).
-template <int N>
-__host__ __device__ constexpr int cols_pass_width() {
-  return (N == 1024 || N == 2048) ? 8 : col_width<N>();
-}
-template <int N>
-__host__ __device__ constexpr int cols_pass_min_blocks() {
-  return FFTConf<N>::T * cols_pass_width<N>() >= 1024 ? 1 : 2;
-}
-
-// Stage twiddles from a shared-memory table (fft.cuh) at N = 2048, where one block per SM leaves
-// room for it; at the other lengths the table would cost resident blocks.
-template <int N>
-__host__ __device__ constexpr int cols_table_size() {
-  return N == 2048 ? stw_size<FFTConf<N>>() : 0;
-}
-
 // In-place FFT of ncols columns per slab: element (n, col) at data[slab*slab_stride + n*row_stride + col].
+// Strips of cols_width columns, two per thread; stage twiddles from shared memory.
 template <int N, bool INV>
-__global__ void __launch_bounds__(FFTConf<N>::T * cols_pass_width<N>(), cols_pass_min_blocks<N>())
+__global__ void __launch_bounds__(cols_threads<N>(), cols_min_blocks<N>())
     k_fft_cols(float2* __restrict__ data, int64_t slab_stride, int64_t row_stride, int ncols,
                const float2* __restrict__ tw) {
   extern __shared__ __align__(16) float2 smem[];
-  constexpr int W = cols_pass_width<N>();
-  if constexpr (cols_table_size<N>() > 0) {
-    float2* stab = smem + N * W;
-    stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, FFTConf<N>::T * W);
-    cols_body<N, W, INV>(data, slab_stride, row_stride, ncols, SmemTw<FFTConf<N>>{stab}, blockIdx.x, blockIdx.y,
-                         smem);
-  } else {
-    cols_body<N, W, INV>(data, slab_stride, row_stride, ncols, tw, blockIdx.x, blockIdx.y, smem);
-  }
+  constexpr int W = cols_width<N>(), SL = cols_slabs<N>();
+  float2* stab = smem + SL * N * W;
+  stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, cols_threads<N>());
+  cols_body<N, W, SL, INV, cpair>(data, slab_stride, row_stride, ncols, SmemTw<FFTConf<N>>{stab}, blockIdx.x,
+                                  blockIdx.y * SL, smem);
 }
 
 // Real rows of length N -> half-spectrum rows (N/2 + 1 entries, stride P), via a complex
@@ -159,18 +137,18 @@ static int x_c2r(const float2* in, float* out, int64_t nrows, int P, const float
 template <int N>
 static int cols(bool inverse, float2* data, int64_t nslabs, int64_t slab_stride, int64_t row_stride, int ncols,
                 const float2* tw, cudaStream_t st) {
-  constexpr int W = cols_pass_width<N>();
-  const size_t smem = (size_t)(N * W + cols_table_size<N>()) * sizeof(float2);
-  if (nslabs > 65535) return fail(COLA_EINVAL, "fft column pass: too many slabs");
-  dim3 grid((ncols + W - 1) / W, (unsigned)nslabs);
+  constexpr int W = cols_width<N>(), SL = cols_slabs<N>();
+  const size_t smem = (size_t)(SL * N * W + stw_size<FFTConf<N>>()) * sizeof(float2);
+  if (nslabs > 65535 || nslabs % SL) return fail(COLA_EINVAL, "fft column pass: unexpected number of slabs");
+  dim3 grid((ncols + W - 1) / W, (unsigned)(nslabs / SL));
   if (inverse) {
     allow_smem(k_fft_cols<N, true>, smem);
     { LaunchScope ls_(label<N>("inv"), st);
-    k_fft_cols<N, true><<<grid, FFTConf<N>::T * W, smem, st>>>(data, slab_stride, row_stride, ncols, tw); }
+    k_fft_cols<N, true><<<grid, cols_threads<N>(), smem, st>>>(data, slab_stride, row_stride, ncols, tw); }
   } else {
     allow_smem(k_fft_cols<N, false>, smem);
     { LaunchScope ls_(label<N>("fwd"), st);
-    k_fft_cols<N, false><<<grid, FFTConf<N>::T * W, smem, st>>>(data, slab_stride, row_stride, ncols, tw); }
+    k_fft_cols<N, false><<<grid, cols_threads<N>(), smem, st>>>(data, slab_stride, row_stride, ncols, tw); }
   }
   COLA_LAUNCH_CHECK();
   return COLA_OK;

@@ -7,6 +7,7 @@
 #include "fft.cuh"
 #include "pm_common.cuh"
 #include "tma.cuh"
+#include "tmem.cuh"
 
 namespace cola {
 
@@ -21,12 +22,38 @@ __device__ __forceinline__ int signed_mode(int k, int n) { return k < n / 2 ? k 
 // first-derivative factor i k_j (zero on the Nyquist plane |n_j| = N/2)
 __device__ __forceinline__ float2 mul_ik(float2 a, float k) { return make_float2(__fmul_rn(-k, a.y), __fmul_rn(k, a.x)); }
 
-// columns per block of the strided passes (16 columns = 128 contiguous bytes per row); blocks
-// of at most 256 threads (512 for the longest transforms) so that two blocks fit on an SM with
-// every thread's E elements in registers, and one block's loads overlap the other's FFT
-template <int N>
-__host__ __device__ constexpr int col_width() {
-  return FFTConf<N>::T * 16 <= 256 ? 16 : (FFTConf<N>::T * 8 <= 256 ? 8 : (FFTConf<N>::T * 4 <= 512 ? 4 : 2));
+// ---- one or two columns per thread ---------------------------------------------------------
+// The strided (column) passes run on strips of W columns, V = float2: one column per thread, V =
+// cpair: two neighbouring columns per thread (fft.cuh).  A half spectrum's rows start on 32-byte
+// boundaries and are padded to a multiple of 4 entries, so the pair that holds the last column
+// (an even one, N/2) has its other lane in the padding, and pairs are 16-byte aligned.
+template <class V>
+__host__ __device__ constexpr int lanes_of() {
+  return (int)(sizeof(V) / sizeof(float2));
+}
+__device__ __forceinline__ cpair c_interleave(float4 q) { return {make_float2(q.x, q.z), make_float2(q.y, q.w)}; }
+__device__ __forceinline__ float4 c_deinterleave(cpair v) { return make_float4(v.re.x, v.im.x, v.re.y, v.im.y); }
+template <class V>
+__device__ __forceinline__ V c_load(const float2* p) {
+  if constexpr (lanes_of<V>() == 1) return *p;
+  else return c_interleave(*reinterpret_cast<const float4*>(p));
+}
+template <class V>
+__device__ __forceinline__ V c_load_cg(const float2* p) {
+  if constexpr (lanes_of<V>() == 1) return __ldcg(p);
+  else return c_interleave(__ldcg(reinterpret_cast<const float4*>(p)));
+}
+template <class V>
+__device__ __forceinline__ V c_zero() {
+  return V{};
+}
+__device__ __forceinline__ void c_store(float2* p, float2 v) { *p = v; }
+__device__ __forceinline__ void c_store(float2* p, cpair v) { *reinterpret_cast<float4*>(p) = c_deinterleave(v); }
+__device__ __forceinline__ void c_store_cg(float2* p, float2 v) { __stcg(p, v); }
+__device__ __forceinline__ void c_store_cg(float2* p, cpair v) { __stcg(reinterpret_cast<float4*>(p), c_deinterleave(v)); }
+// first-derivative factor i k of both lanes
+__device__ __forceinline__ cpair mul_ik(cpair a, float k) {
+  return {p_mul_rn(p_dup(-k), a.im), p_mul_rn(p_dup(k), a.re)};
 }
 
 // row pitch (complex entries) of a half spectrum of an N^3 mesh: N/2 + 1 rounded up to a multiple
@@ -36,22 +63,98 @@ __host__ __device__ constexpr int half_pitch() {
   return ((N / 2 + 1) + 3) / 4 * 4;
 }
 
-// block (bx, slab): W columns of one slab of the in-place strided FFT (T(N) * W threads);
-// smem: N W float2.  Element (n, col) at data[slab * slab_stride + n * row_stride + col].
+// Strip width (columns per block), slabs per block, threads and resident blocks per SM of the
+// single-box column passes, two columns per thread: 16 columns are 128-byte row segments, 8 where
+// a strip of 16 would leave room for fewer than two blocks in shared memory.  The registers of E
+// complex pairs (4 E) set the threads per SM.
+template <int N>
+__host__ __device__ constexpr int cols_width() {
+  return N >= 512 ? 8 : 16;
+}
+// two slabs per block where one makes a block of one or two warps whose parked words take a
+// quarter of the tensor memory
+template <int N>
+__host__ __device__ constexpr int cols_slabs() {
+  return N == 192 || N == 96 ? 2 : 1;
+}
+template <int N>
+__host__ __device__ constexpr int cols_threads() {
+  return FFTConf<N>::T * cols_width<N>() / 2 * cols_slabs<N>();
+}
+template <int N>
+__host__ __device__ constexpr int cols_min_blocks() {
+  constexpr int E = FFTConf<N>::E, threads = cols_threads<N>();
+  constexpr int per_sm = (E >= 24 ? 384 : (E >= 12 ? 512 : 768)) / threads;
+  // (and no more blocks than have their parked words in the tensor memory at once)
+  constexpr int parked = 512 / tmem_columns(threads, (4 * E + 15) / 16 * 16);
+  return per_sm < 1 ? 1 : (per_sm < parked ? per_sm : parked);
+}
+// one thread's E elements, parked (tmem.cuh)
+template <int THREADS, int E, class V>
+using Park = TmemPark<THREADS, (E * lanes_of<V>() * 2 + 15) / 16 * 16>;
+template <class P, int E, class V>
+__device__ __forceinline__ void park_store(const P& park, const V (&u)[E]) {
+  uint32_t r[(sizeof(u) / 4 + 15) / 16 * 16] = {};
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    if constexpr (lanes_of<V>() == 1) {
+      r[2 * m] = __float_as_uint(u[m].x);
+      r[2 * m + 1] = __float_as_uint(u[m].y);
+    } else {
+      r[4 * m] = __float_as_uint(u[m].re.x);
+      r[4 * m + 1] = __float_as_uint(u[m].re.y);
+      r[4 * m + 2] = __float_as_uint(u[m].im.x);
+      r[4 * m + 3] = __float_as_uint(u[m].im.y);
+    }
+  }
+  park.store(r);
+}
+template <class P, int E, class V>
+__device__ __forceinline__ void park_load(const P& park, V (&u)[E]) {
+  uint32_t r[(sizeof(u) / 4 + 15) / 16 * 16];
+  park.load(r);
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    if constexpr (lanes_of<V>() == 1)
+      u[m] = make_float2(__uint_as_float(r[2 * m]), __uint_as_float(r[2 * m + 1]));
+    else
+      u[m] = V{make_float2(__uint_as_float(r[4 * m]), __uint_as_float(r[4 * m + 1])),
+               make_float2(__uint_as_float(r[4 * m + 2]), __uint_as_float(r[4 * m + 3]))};
+  }
+}
+
+// This thread's place in a block that takes W columns of each of SL slabs: columns w K .. of the
+// strip, transform thread t, slab number sub; strips of the exchange buffer slab after slab.
+template <int N, int W, int SL, class V, class C>
+struct ColsThread {
+  static constexpr int K = lanes_of<V>(), WT = W / K, T = C::T, NT = T * WT * SL;
+  int w, t, sub;
+  V* S;
+  __device__ __forceinline__ explicit ColsThread(float2* smem) {
+    const int i = threadIdx.x;
+    w = i % WT;
+    t = i / WT % T;
+    sub = SL == 1 ? 0 : i / (WT * T);
+    S = reinterpret_cast<V*>(smem) + (SL == 1 ? 0 : sub * (N * WT));
+  }
+  __device__ __forceinline__ V& operator()(int n) const { return S[n * WT + w]; }
+};
+
+// block (bx, slab0): W columns of SL slabs of the in-place strided FFT (T(N) * W / lanes * SL
+// threads); smem: SL N W float2.  Element (n, col) at data[slab * slab_stride + n * row_stride + col].
 // (tw: the base twiddle table or an SmemTw stage table)
-template <int N, int W, bool INV, class C = FFTConf<N>, class TW>
+template <int N, int W, int SL, bool INV, class V, class C = FFTConf<N>, class TW>
 __device__ __forceinline__ void cols_body(float2* __restrict__ data, int64_t slab_stride, int64_t row_stride,
-                                          int ncols, const TW& tw, int bx, int slab, float2* smem) {
-  const int w = threadIdx.x % W, t = threadIdx.x / W;
-  const int col = bx * W + w;
+                                          int ncols, const TW& tw, int bx, int slab0, float2* smem) {
+  const ColsThread<N, W, SL, V, C> mem(smem);
+  const int col = bx * W + mem.w * mem.K;
   const bool valid = col < ncols;
-  float2* base = data + (int64_t)slab * slab_stride + (valid ? col : 0);
-  auto load = [&](int n) -> float2 { return valid ? base[(int64_t)n * row_stride] : make_float2(0.f, 0.f); };
-  auto mem = [&](int n) -> float2& { return smem[n * W + w]; };
-  auto store = [&](int n, float2 x) {
-    if (valid) base[(int64_t)n * row_stride] = x;
+  float2* base = data + (int64_t)(slab0 + mem.sub) * slab_stride + (valid ? col : 0);
+  auto load = [&](int n) -> V { return valid ? c_load<V>(base + (int64_t)n * row_stride) : c_zero<V>(); };
+  auto store = [&](int n, V x) {
+    if (valid) c_store(base + (int64_t)n * row_stride, x);
   };
-  fft_1d<N, 1, INV, C>(t, tw, load, mem, store);
+  fft_1d<N, 1, INV, C>(mem.t, tw, load, mem, store);
 }
 
 // ---- 1. deposit + x r2c -----------------------------------------------------------------------
@@ -183,309 +286,152 @@ __device__ __forceinline__ void deposit_fftx_body(const Geometry& g, const Tiles
 }
 
 // ---- 3. z pass with the Green's function ------------------------------------------------------------
-// block (bx, ky): W columns kx of the slab ky (T(N) * W threads); sm: 2 N W float2
-// (stw: the stage twiddles, the base table tw or an SmemTw table)
-template <int N, int W, class C = FFTConf<N>, class STW>
-__device__ __forceinline__ void z_green_body(float2* __restrict__ A, float2* __restrict__ Gz, int P, float kf,
-                                             int deconv, float norm, const STW& stw, int bx, int ky, float2* sm) {
-  constexpr int nh = N / 2 + 1, NT = C::T * W;
-  float2* S0 = sm;           // delta_k of the slab, [n][W]
-  float2* S1 = sm + N * W;   // exchange buffer
-  const int w = threadIdx.x % W, t = threadIdx.x / W;
-  const int kx = bx * W + w;
-  const bool valid = kx < nh;
-  const int64_t zstride = (int64_t)N * P;
-  float2* a = A + (int64_t)ky * P + (valid ? kx : 0);
-  float2* gz = Gz + (int64_t)ky * P + (valid ? kx : 0);
-  auto mem = [&](int n) -> float2& { return S1[n * W + w]; };
-  {
-    auto load = [&](int n) -> float2 { return valid ? a[n * zstride] : make_float2(0.f, 0.f); };
-    auto store = [&](int n, float2 x) { S0[n * W + w] = x; };
-    fft_1d<N, 1, false, C>(t, stw, load, mem, store);
+// Forward transform of the strip, phi = delta_k norm / (k^2 W(k)^p), then the inverse transforms
+// of i k_z phi (-> Gz) and of phi (-> A, in place): one load and two stores of the strip.  A
+// thread ends a transform with the elements the next one starts from, so phi stays in its
+// registers and its second use is parked in tensor memory.
+//
+// shared-memory layout: SL strips (N W float2 each), sinc^2 tables (N + W floats, rounded up to
+// 16 bytes), stage twiddle table
+template <int N, int W, int SL>
+__host__ __device__ constexpr int z_table_offset() {
+  return SL * N * W + (N + W + 3) / 4 * 2;
+}
+
+// norm / (kf2 m2 W^p): the Green's function of one mode (wk = W(k))
+__device__ __forceinline__ float green_of(int m2, float kf2, float wk, int deconv, float norm) {
+  float gk = 0.0f;
+  if (m2 != 0) {
+    float den = kf2 * (float)m2;
+    if (deconv) den *= deconv == 2 ? wk * wk : wk;
+    gk = __fdividef(norm, den);  // fast reciprocal: <= 2 ulp, far below the transforms' rounding
   }
-  // sinc^2 tables of the z index and of the block's W columns, then
-  // phi_k = delta_k norm / (k^2 W(k)^p) in place in S0 with one division per mode
-  float* sz2 = reinterpret_cast<float*>(S1);  // S1 is free between the transforms
+  return gk;
+}
+
+// block (bx, ky0): W columns kx of SL slabs ky (T(N) W / lanes SL threads)
+template <int N, int W, int SL, class V, class C = FFTConf<N>, class P_>
+__device__ __forceinline__ void z_green_body(float2* __restrict__ A, float2* __restrict__ Gz, float kf, int deconv,
+                                             float norm, const float2* __restrict__ tw, int bx, int ky0, float2* sm,
+                                             const P_& park) {
+  constexpr int K = lanes_of<V>(), E = C::E, T = C::T, nh = N / 2 + 1, P = half_pitch<N>();
+  const ColsThread<N, W, SL, V, C> mem(sm);
+  float* sz2 = reinterpret_cast<float*>(sm + SL * N * W);
   float* sx2 = sz2 + N;
-  for (int n = threadIdx.x; n < N + W; n += NT) {
+  float2* stab = sm + z_table_offset<N, W, SL>();
+  stw_fill<C, 1>(stab, tw, threadIdx.x, mem.NT);
+  const SmemTw<C> stw{stab};
+  const int t = mem.t, ky = ky0 + mem.sub;
+  const int kx = bx * W + mem.w * K;
+  const bool valid = kx < nh;
+  constexpr int64_t zstride = (int64_t)N * P;
+  const int64_t at = (int64_t)ky * P + (valid ? kx : 0) + t * zstride;
+  float2* a = A + at;
+  float2* gz = Gz + at;
+  V u[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) u[m] = valid ? c_load<V>(a + m * (T * zstride)) : c_zero<V>();
+  for (int n = threadIdx.x; n < N + W; n += mem.NT) {
     const float sv = n < N ? sinc_pi_f(signed_mode(n, N), N) : sinc_pi_f(bx * W + (n - N), N);
     (n < N ? sz2[n] : sx2[n - N]) = sv * sv;
   }
-  __syncthreads();
+  fft_regs<N, 1, false, C>(u, t, stw, mem);
   {
     const int ny = signed_mode(ky, N);
     const float sy = sinc_pi_f(ny, N);
     const float wy = sy * sy;
     const float kf2 = kf * kf;
-    for (int i = threadIdx.x; i < N * W; i += NT) {
-      const int n = i / W, c = i - n * W;
-      const int nx = bx * W + c;
-      const int nz = signed_mode(n, N);
-      const int m2 = nx * nx + ny * ny + nz * nz;
-      float gk = 0.0f;
-      if (m2 != 0 && nx < nh) {
-        float den = kf2 * (float)m2;
-        if (deconv) {
-          const float wk = sx2[c] * wy * sz2[n];
-          den *= deconv == 2 ? wk * wk : wk;
-        }
-        gk = __fdividef(norm, den);  // fast reciprocal: <= 2 ulp, far below the transforms' rounding
+    const float wxy0 = sx2[mem.w * K] * wy, wxy1 = sx2[mem.w * K + K - 1] * wy;
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int n = t + T * m, nz = signed_mode(n, N);
+      const int myz = ny * ny + nz * nz;
+      const float s0 = green_of(kx * kx + myz, kf2, wxy0 * sz2[n], deconv, norm);
+      if constexpr (K == 1) {
+        u[m] = c_scale(u[m], s0);
+      } else {
+        const float s1 = green_of((kx + 1) * (kx + 1) + myz, kf2, wxy1 * sz2[n], deconv, norm);
+        u[m] = c_scale(u[m], make_float2(s0, s1));
       }
-      S0[i] = c_scale(S0[i], gk);
     }
   }
-  __syncthreads();
-  {
-    auto load = [&](int n) -> float2 { return S0[n * W + w]; };
-    auto store = [&](int n, float2 x) {
-      if (valid) a[n * zstride] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
+  park_store(park, u);
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int n = t + T * m;
+    u[m] = mul_ik(u[m], (n == N / 2) ? 0.0f : kf * (float)signed_mode(n, N));
   }
-  {
-    auto load = [&](int n) -> float2 {
-      const float kz = (n == N / 2) ? 0.0f : kf * (float)signed_mode(n, N);
-      return mul_ik(S0[n * W + w], kz);
-    };
-    auto store = [&](int n, float2 x) {
-      if (valid) gz[n * zstride] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
+  fft_regs<N, 1, true, C>(u, t, stw, mem);
+  if (valid) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) c_store(gz + m * (T * zstride), u[m]);
   }
+  __syncwarp();
+  park_load(park, u);
+  fft_regs<N, 1, true, C>(u, t, stw, mem);
+  if (valid) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) c_store(a + m * (T * zstride), u[m]);
+  }
+  __syncwarp();
 }
 
 // ---- 4. inverse y passes ------------------------------------------------------------------------------------
-// block (bx, z): W columns kx of the slab z (T(N) * W threads); sm: 2 N W float2
-template <int N, int W, class C = FFTConf<N>, class STW>
+// Gy = IFFT_y(i k_y B), then B = IFFT_y(B) in place, then Gz = IFFT_y(Gz): the strip of B is read
+// once and parked in tensor memory for its second transform.  block (bx, z0): W columns kx of SL
+// slabs z (T(N) W / lanes SL threads); sm: SL N W float2, then the stage twiddle table
+template <int N, int W, int SL, class V, class C = FFTConf<N>, class P_>
 __device__ __forceinline__ void y_inv3_body(float2* __restrict__ B, float2* __restrict__ Gy, float2* __restrict__ Gz,
-                                            int P, float kf, const STW& stw, int bx, int z, float2* sm) {
-  constexpr int nh = N / 2 + 1, T = C::T;
-  float2* S0 = sm;
-  float2* S1 = sm + N * W;
-  const int w = threadIdx.x % W, t = threadIdx.x / W;
-  const int kx = bx * W + w;
-  const bool valid = kx < nh;
-  const int64_t slab = (int64_t)z * N * P + (valid ? kx : 0);
-  float2* b = B + slab;
-  float2* gy = Gy + slab;
-  float2* gz = Gz + slab;
-  // the Gz strip is read only by the third transform: start pulling it into L2 now
-  if (w == 0)
-    for (int n = t; n < N; n += T) prefetch_l2_line(Gz + (int64_t)z * N * P + bx * W + (int64_t)n * P);
-  for (int n = t; n < N; n += T) S0[n * W + w] = valid ? b[(int64_t)n * P] : make_float2(0.f, 0.f);
-  __syncthreads();
-  auto mem = [&](int n) -> float2& { return S1[n * W + w]; };
-  {
-    auto load = [&](int n) -> float2 { return S0[n * W + w]; };
-    auto store = [&](int n, float2 x) {
-      if (valid) b[(int64_t)n * P] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
-  }
-  {
-    auto load = [&](int n) -> float2 {
-      const float ky = (n == N / 2) ? 0.0f : kf * (float)signed_mode(n, N);
-      return mul_ik(S0[n * W + w], ky);
-    };
-    auto store = [&](int n, float2 x) {
-      if (valid) gy[(int64_t)n * P] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
-  }
-  {
-    auto load = [&](int n) -> float2 { return valid ? gz[(int64_t)n * P] : make_float2(0.f, 0.f); };
-    auto store = [&](int n, float2 x) {
-      if (valid) gz[(int64_t)n * P] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
-  }
-}
-
-// ---- 3'/4'. single-buffer (wide-strip) variants of the z and inverse y passes ------------------------------
-// For long columns the two-buffer bodies above leave room for only narrow strips (4 columns =
-// 32-byte row segments at N = 2048).  These variants keep one exchange buffer of N x W complex
-// and re-read their input strip from global memory (an L2 hit) for each transform instead of
-// holding it in shared memory, so the strips can be twice as wide.
-//
-// z pass: forward transform of the strip, phi = delta_k norm / (k^2 W(k)^p) written back to A in
-// the forward transform's last stage, then the inverse transforms of i k_z phi (-> Gz) and of phi
-// (-> A, in place).  block (bx, ky): W columns kx of the slab ky (T(N) * W threads);
-// sm: N W float2 + (N + W) floats (sinc^2 tables).
-// shared-memory layout of the wide z pass: strip (N W float2), sinc^2 tables (N + W floats,
-// rounded up to 16 bytes), stage twiddle table
-template <int N, int W>
-__host__ __device__ constexpr int wide_z_table_offset() {
-  return N * W + (N + W + 3) / 4 * 2;
-}
-// scratch slots of the wide z pass (one per SM id, N W float2 each)
-constexpr int kZScratchSlots = 512;
-
-// z pass with the Green's function, one exchange buffer.  With KS > 0 scratch slots per SM the
-// forward transform of the strip (Green's function applied as it is stored) goes to a slot of
-// this SM, contiguous [n][w], and the inverse transforms of i k_z phi (-> Gz) and of phi (-> A)
-// read it back from L2 as whole 128-byte lines (the strip itself spans N rows N (N/2+1) 8 bytes
-// apart: 16.8 MB at N = 2048).  KS = 1: one block fits per SM (shared memory), so the slot of
-// %smid is the block's own while it runs; KS > 1: a block claims one of its SM's KS slots
-// (compare-and-swap on busy[], a bounded number of rounds) and frees it when it is done, KS
-// being above the blocks that fit on an SM.  KS = 0: phi goes to A and the inverse transforms
-// read it back from there (an L2 hit).
-// block (bx, ky): W columns kx of the slab ky (T(N) W threads); scratch: kZScratchSlots KS N W
-// float2; busy: kZScratchSlots KS ints, zero between launches
-template <int N, int W, int KS, class C = FFTConf<N>>
-__device__ __forceinline__ void z_green_wide_body(float2* __restrict__ A, float2* __restrict__ Gz,
-                                                  float2* __restrict__ scratch, int* __restrict__ busy, float kf,
-                                                  int deconv, float norm, const float2* __restrict__ tw,
-                                                  int* __restrict__ err, int bx, int ky, float2* sm) {
-  constexpr int nh = N / 2 + 1, NT = C::T * W, P = half_pitch<N>();
-  constexpr bool SCRATCH = KS > 0;
-  float2* sc = nullptr;
-  int* my_flag = nullptr;
-  if constexpr (SCRATCH) {
-    unsigned smid, nsmid;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-    asm volatile("mov.u32 %0, %%nsmid;" : "=r"(nsmid));
-    if (nsmid > (unsigned)kZScratchSlots) {
-      if (threadIdx.x == 0) atomicOr(err, kErrSmIds);
-      return;
-    }
-    int slot = (int)smid * KS;
-    if constexpr (KS > 1) {
-      __shared__ int claimed;
-      if (threadIdx.x == 0) {
-        int got = -1;
-        for (int round = 0; round < 1024 && got < 0; ++round)
-          for (int k = 0; k < KS && got < 0; ++k)
-            if (atomicCAS(busy + slot + k, 0, 1) == 0) got = k;
-        claimed = got;
-      }
-      __syncthreads();
-      if (claimed < 0) {
-        if (threadIdx.x == 0) atomicOr(err, kErrSmIds);
-        return;
-      }
-      slot += claimed;
-      my_flag = busy + slot;
-    }
-    sc = scratch + (int64_t)slot * (N * W);
-  }
-  float2* S = sm;
-  float* sz2 = reinterpret_cast<float*>(sm + N * W);
-  float* sx2 = sz2 + N;
-  float2* stab = sm + wide_z_table_offset<N, W>();
-  stw_fill<C, 1>(stab, tw, threadIdx.x, NT);
+                                            float kf, const float2* __restrict__ tw, int bx, int z0, float2* sm,
+                                            const P_& park) {
+  constexpr int K = lanes_of<V>(), E = C::E, T = C::T, nh = N / 2 + 1, P = half_pitch<N>();
+  const ColsThread<N, W, SL, V, C> mem(sm);
+  float2* stab = sm + SL * N * W;
+  stw_fill<C, 1>(stab, tw, threadIdx.x, mem.NT);
   const SmemTw<C> stw{stab};
-  const int w = threadIdx.x % W, t = threadIdx.x / W;
-  const int kx = bx * W + w;
+  const int t = mem.t;
+  const int kx = bx * W + mem.w * K;
   const bool valid = kx < nh;
-  constexpr int64_t zstride = (int64_t)N * P;
-  float2* a = A + (int64_t)ky * P + (valid ? kx : 0);
-  float2* gz = Gz + (int64_t)ky * P + (valid ? kx : 0);
-  for (int n = threadIdx.x; n < N + W; n += NT) {
-    const float sv = n < N ? sinc_pi_f(signed_mode(n, N), N) : sinc_pi_f(bx * W + (n - N), N);
-    (n < N ? sz2[n] : sx2[n - N]) = sv * sv;
-  }
-  if constexpr (SCRATCH) {
-    // the slot still holds the previous block's strip, dead now: drop its lines from L2 rather
-    // than let them be written back (the barrier orders this before the slot's new writes)
-    for (int l = threadIdx.x; l < N * W * (int)sizeof(float2) / 128; l += NT)
-      discard_l2_line(reinterpret_cast<char*>(sc) + 128 * l);
-  }
-  __syncthreads();
-  // phi of element n of this thread's column: where the forward transform leaves it
-  auto phi_at = [&](int n) -> float2* { return SCRATCH ? sc + n * W + w : a + n * zstride; };
-  auto mem = [&](int n) -> float2& { return S[n * W + w]; };
-  {
-    const int ny = signed_mode(ky, N);
-    const float sy = sinc_pi_f(ny, N);
-    const float wy = sy * sy;
-    const float kf2 = kf * kf;
-    auto load = [&](int n) -> float2 { return valid ? a[n * zstride] : make_float2(0.f, 0.f); };
-    auto store = [&](int n, float2 x) {
-      const int nz = signed_mode(n, N);
-      const int m2 = kx * kx + ny * ny + nz * nz;
-      float gk = 0.0f;
-      if (m2 != 0) {
-        float den = kf2 * (float)m2;
-        if (deconv) {
-          const float wk = sx2[w] * wy * sz2[n];
-          den *= deconv == 2 ? wk * wk : wk;
-        }
-        gk = __fdividef(norm, den);
-      }
-      if (SCRATCH || valid) __stcg(phi_at(n), c_scale(x, gk));
-    };
-    fft_1d<N, 1, false, C>(t, stw, load, mem, store);
-  }
-  __syncthreads();  // phi of the strip is in the scratch slot or in A (visible to the block after the barrier)
-  {
-    auto load = [&](int n) -> float2 {
-      const float kz = (n == N / 2) ? 0.0f : kf * (float)signed_mode(n, N);
-      return (SCRATCH || valid) ? mul_ik(__ldcg(phi_at(n)), kz) : make_float2(0.f, 0.f);
-    };
-    auto store = [&](int n, float2 x) {
-      if (valid) gz[n * zstride] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
-  }
-  {
-    auto load = [&](int n) -> float2 { return (SCRATCH || valid) ? __ldcg(phi_at(n)) : make_float2(0.f, 0.f); };
-    auto store = [&](int n, float2 x) {
-      if (valid) a[n * zstride] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
-  }
-  if constexpr (KS > 1) {
-    __syncthreads();  // every read of the slot is done: free it (the exchange returns when done)
-    if (threadIdx.x == 0) atomicExch(my_flag, 0);
-  }
-}
-
-// inverse y passes, one exchange buffer: Gy = IFFT_y(i k_y B), then B = IFFT_y(B) in place (the
-// strip of B read again, from L2), then Gz = IFFT_y(Gz).  block (bx, z): W columns kx of the slab
-// z (T(N) * W threads); sm: N W float2
-template <int N, int W, class C = FFTConf<N>>
-__device__ __forceinline__ void y_inv3_wide_body(float2* __restrict__ B, float2* __restrict__ Gy,
-                                                 float2* __restrict__ Gz, float kf, const float2* __restrict__ tw,
-                                                 int bx, int z, float2* sm) {
-  constexpr int nh = N / 2 + 1, T = C::T, P = half_pitch<N>();
-  float2* stab = sm + N * W;
-  stw_fill<C, 1>(stab, tw, threadIdx.x, T * W);
-  const SmemTw<C> stw{stab};
-  const int w = threadIdx.x % W, t = threadIdx.x / W;
-  const int kx = bx * W + w;
-  const bool valid = kx < nh;
-  const int64_t slab = (int64_t)z * N * P + (valid ? kx : 0);
-  float2* b = B + slab;
-  float2* gy = Gy + slab;
-  float2* gz = Gz + slab;
+  const int64_t at = (int64_t)(z0 + mem.sub) * N * P + (valid ? kx : 0) + t * P;
+  float2* b = B + at;
+  float2* gy = Gy + at;
+  float2* gz = Gz + at;
+  V u[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) u[m] = valid ? c_load<V>(b + m * (T * P)) : c_zero<V>();
   // the Gz strip is read only by the third transform: start pulling it into L2 now
-  if (w == 0)
-    for (int n = t; n < N; n += T) prefetch_l2_line(Gz + (int64_t)z * N * P + bx * W + (int64_t)n * P);
-  auto mem = [&](int n) -> float2& { return sm[n * W + w]; };
-  {
-    auto load = [&](int n) -> float2 {
-      const float ky = (n == N / 2) ? 0.0f : kf * (float)signed_mode(n, N);
-      return valid ? mul_ik(b[(int64_t)n * P], ky) : make_float2(0.f, 0.f);
-    };
-    auto store = [&](int n, float2 x) {
-      if (valid) gy[(int64_t)n * P] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
+  if (mem.w == 0 && valid) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) prefetch_l2_line(gz + m * (T * P));
   }
-  {
-    auto load = [&](int n) -> float2 { return valid ? b[(int64_t)n * P] : make_float2(0.f, 0.f); };
-    auto store = [&](int n, float2 x) {
-      if (valid) b[(int64_t)n * P] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
+  __syncwarp();
+  park_store(park, u);
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int n = t + T * m;
+    u[m] = mul_ik(u[m], (n == N / 2) ? 0.0f : kf * (float)signed_mode(n, N));
   }
-  {
-    auto load = [&](int n) -> float2 { return valid ? gz[(int64_t)n * P] : make_float2(0.f, 0.f); };
-    auto store = [&](int n, float2 x) {
-      if (valid) gz[(int64_t)n * P] = x;
-    };
-    fft_1d<N, 1, true, C>(t, stw, load, mem, store);
+  fft_regs<N, 1, true, C>(u, t, stw, mem);
+  if (valid) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) c_store(gy + m * (T * P), u[m]);
   }
+  __syncwarp();
+  park_load(park, u);
+  fft_regs<N, 1, true, C>(u, t, stw, mem);
+  if (valid) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) c_store(b + m * (T * P), u[m]);
+#pragma unroll
+    for (int m = 0; m < E; ++m) u[m] = c_load<V>(gz + m * (T * P));
+  }
+  __syncwarp();
+  fft_regs<N, 1, true, C>(u, t, stw, mem);
+  if (valid) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) c_store(gz + m * (T * P), u[m]);
+  }
+  __syncwarp();
 }
 
 // ---- 5. inverse x passes of the three components -------------------------------------------------------------

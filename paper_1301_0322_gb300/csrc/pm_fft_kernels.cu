@@ -54,87 +54,33 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * TY * TZ, deposit_min_block
 }
 
 template <int N>
-__global__ void __launch_bounds__(FFTConf<N>::T * col_width<N>(), 2)
-    k_fft_z_green(float2* __restrict__ A, float2* __restrict__ Gz, int P, float kf, int deconv, float norm,
+using ColsPark = Park<cols_threads<N>(), FFTConf<N>::E, cpair>;
+template <int N>
+__global__ void __launch_bounds__(cols_threads<N>(), cols_min_blocks<N>())
+    k_fft_z_green(float2* __restrict__ A, float2* __restrict__ Gz, float kf, int deconv, float norm,
                   const float2* __restrict__ tw) {
-  extern __shared__ float2 sm[];
-  z_green_body<N, col_width<N>()>(A, Gz, P, kf, deconv, norm, tw, blockIdx.x, blockIdx.y, sm);
+  extern __shared__ __align__(16) float2 sm[];
+  __shared__ uint32_t slot;
+  const ColsPark<N> park(&slot);
+  constexpr int SL = cols_slabs<N>();
+  z_green_body<N, cols_width<N>(), SL, cpair>(A, Gz, kf, deconv, norm, tw, blockIdx.x, blockIdx.y * SL, sm, park);
+  park.close();
+}
+template <int N>
+constexpr size_t z_smem() {
+  return sizeof(float2) * (z_table_offset<N, cols_width<N>(), cols_slabs<N>()>() + stw_size<FFTConf<N>>());
 }
 
 template <int N>
-__global__ void __launch_bounds__(FFTConf<N>::T * col_width<N>(), 2)
-    k_fft_y_inv3(float2* __restrict__ B, float2* __restrict__ Gy, float2* __restrict__ Gz, int P, float kf,
+__global__ void __launch_bounds__(cols_threads<N>(), cols_min_blocks<N>())
+    k_fft_y_inv3(float2* __restrict__ B, float2* __restrict__ Gy, float2* __restrict__ Gz, float kf,
                  const float2* __restrict__ tw) {
-  extern __shared__ float2 sm[];
-  y_inv3_body<N, col_width<N>()>(B, Gy, Gz, P, kf, tw, blockIdx.x, blockIdx.y, sm);
-}
-
-// Strip widths of the single-buffer (wide-strip) z, forward y and inverse y passes, 0 where the
-// two-buffer bodies (z, inverse y) or the stand-alone column pass (forward y) are used.  At 256,
-// 16-column strips: z 0.88 -> 0.75, forward y 0.34 -> 0.31 ms per 128^3/256^3 run; at 768 the
-// stand-alone forward y pass stays faster.
-template <int N>
-__host__ __device__ constexpr int wide_width() {
-  return (N == 2048 || N == 768) ? 8 : ((N >= 128 && N <= 256) ? 16 : 0);
-}
-template <int N>
-__host__ __device__ constexpr int wide_fwd_width() {
-  return N == 768 ? 0 : wide_width<N>();
-}
-// the same for the inverse y passes (768: 27.0 -> 23.5 ms per 256^3/768^3 run; 16-column strips
-// at 128-256: 1.43 -> 0.75 ms per 128^3/256^3 run)
-template <int N>
-__host__ __device__ constexpr int wide_inv_width() {
-  return (N == 2048 || N == 768) ? 8 : ((N >= 128 && N <= 256) ? 16 : 0);
-}
-template <int N, int W>
-__host__ __device__ constexpr int wide_min_blocks() {
-  return FFTConf<N>::T * W >= 1024 ? 1 : 2;
-}
-
-// scratch slots per SM of the wide z pass: the SM's own slot where one block fits (2048), four
-// claimed slots at 768 (at most three blocks of 58 KB fit), none elsewhere
-template <int N, int W>
-__host__ __device__ constexpr int wide_z_slots() {
-  return wide_min_blocks<N, W>() == 1 ? 1 : (N == 768 ? 4 : 0);
-}
-// slot flags of the claimed scratch slots (zero between launches: every block frees its slot)
-__device__ int g_zslot_busy[kZScratchSlots * 4];
-
-template <int N, int W>
-__global__ void __launch_bounds__(FFTConf<N>::T * W, wide_min_blocks<N, W>())
-    k_fft_z_green_wide(float2* __restrict__ A, float2* __restrict__ Gz, float2* __restrict__ scratch, float kf,
-                       int deconv, float norm, const float2* __restrict__ tw, int* __restrict__ err) {
   extern __shared__ __align__(16) float2 sm[];
-  z_green_wide_body<N, W, wide_z_slots<N, W>()>(A, Gz, scratch, g_zslot_busy, kf, deconv, norm, tw, err,
-                                                 blockIdx.x, blockIdx.y, sm);
-}
-// the scratch slot of an SM belongs to one block only if two blocks cannot share the SM
-template <int N, int W>
-constexpr size_t wide_z_smem() {
-  return sizeof(float2) * (wide_z_table_offset<N, W>() + stw_size<FFTConf<N>>());
-}
-static_assert(2 * wide_z_smem<2048, 8>() > 228 * 1024, "two wide z blocks would fit on one SM");
-static_assert(4 * (wide_z_smem<768, 8>() + 1024) > 228 * 1024, "four wide z blocks would fit on one SM");
-
-template <int N, int W>
-__global__ void __launch_bounds__(FFTConf<N>::T * W, wide_min_blocks<N, W>())
-    k_fft_y_inv3_wide(float2* __restrict__ B, float2* __restrict__ Gy, float2* __restrict__ Gz, float kf,
-                      const float2* __restrict__ tw) {
-  extern __shared__ __align__(16) float2 sm[];
-  y_inv3_wide_body<N, W>(B, Gy, Gz, kf, tw, blockIdx.x, blockIdx.y, sm);
-}
-
-// forward y pass of the half spectrum in strips of W columns (slab = z)
-template <int N, int W>
-__global__ void __launch_bounds__(FFTConf<N>::T * W, wide_min_blocks<N, W>())
-    k_fft_y_fwd_wide(float2* __restrict__ A, const float2* __restrict__ tw) {
-  extern __shared__ __align__(16) float2 sm[];
-  constexpr int P = half_pitch<N>();
-  float2* stab = sm + N * W;
-  stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, FFTConf<N>::T * W);
-  const SmemTw<FFTConf<N>> stw{stab};
-  cols_body<N, W, false>(A, (int64_t)N * P, P, N / 2 + 1, stw, blockIdx.x, blockIdx.y, sm);
+  __shared__ uint32_t slot;
+  const ColsPark<N> park(&slot);
+  constexpr int SL = cols_slabs<N>();
+  y_inv3_body<N, cols_width<N>(), SL, cpair>(B, Gy, Gz, kf, tw, blockIdx.x, blockIdx.y * SL, sm, park);
+  park.close();
 }
 
 // Persistent: each block walks items blockIdx.x, blockIdx.x + gridDim.x, ... with the bulk
@@ -211,11 +157,10 @@ static int set_smem(K kernel, size_t bytes) {
 
 template <int N>
 static const char* flabel(int kind) {
-  static const std::string names[5] = {std::string("deposit_fftx_") + std::to_string(N),
+  static const std::string names[4] = {std::string("deposit_fftx_") + std::to_string(N),
                                        std::string("fft_z_green_") + std::to_string(N),
                                        std::string("fft_y_inv3_") + std::to_string(N),
-                                       std::string("fft_x_c2r3_") + std::to_string(N),
-                                       std::string("fft_cols_fwd_") + std::to_string(N)};
+                                       std::string("fft_x_c2r3_") + std::to_string(N)};
   return names[kind].c_str();
 }
 
@@ -246,78 +191,34 @@ static int deposit_fftx_t(const Geometry& g, const Tiles& tl, const uint4* rec, 
   return COLA_OK;
 }
 
-// 2. forward y pass of the half spectrum A
-template <int N>
-static int forward_y_t(float2* A, int P, const float2* tw, cudaStream_t st) {
-  constexpr int nh = N / 2 + 1, WF = wide_fwd_width<N>();
-  if constexpr (WF > 0) {
-    if (P != half_pitch<N>()) return fail(COLA_EINVAL, "wide column passes: unexpected half-spectrum pitch");
-    int rc;
-    const dim3 grid((nh + WF - 1) / WF, N);
-    const size_t smem = sizeof(float2) * (N * WF + stw_size<FFTConf<N>>());
-    if ((rc = set_smem(k_fft_y_fwd_wide<N, WF>, smem))) return rc;
-    LaunchScope ls_(flabel<N>(4), st);
-    k_fft_y_fwd_wide<N, WF><<<grid, FFTConf<N>::T * WF, smem, st>>>(A, tw);
-    COLA_LAUNCH_CHECK();
-    return COLA_OK;
-  } else {
-    return launch_fft_cols(N, false, A, N, (int64_t)N * P, P, nh, tw, st);
-  }
-}
-
 template <int N>
 static int force_passes_t(const Geometry& g, const Tiles& tl, const uint4* rec, const int* offsets,
                           float2* A, float2* Gy, float2* Gz, float* F, int P, double box, int deconv,
                           const float2* tw, int* err, cudaStream_t st) {
-  constexpr int M = N / 2, W = col_width<N>(), nh = N / 2 + 1;
+  constexpr int M = N / 2, W = cols_width<N>(), nh = N / 2 + 1;
   const float kf = (float)(2.0 * 3.14159265358979323846 / box);
   const float norm = (float)(1.0 / ((double)N * N * N));
+  if (P != half_pitch<N>()) return fail(COLA_EINVAL, "force passes: unexpected half-spectrum pitch");
   int rc;
   if ((rc = deposit_fftx_t<N>(g, tl, rec, offsets, A, P, tw, err, st))) return rc;
-  constexpr int WW = wide_width<N>(), WI = wide_inv_width<N>();
-  if constexpr (WW > 0 || WI > 0) {
-    if (P != half_pitch<N>()) return fail(COLA_EINVAL, "wide column passes: unexpected half-spectrum pitch");
-  }
-  if ((rc = forward_y_t<N>(A, P, tw, st))) return rc;
-  if constexpr (WW > 0) {
-    const dim3 grid((nh + WW - 1) / WW, N);
-    constexpr int NT = FFTConf<N>::T * WW;
-    // 3. z pass with the Green's function; its scratch slots sit at the start of Gy, which the
-    // inverse y passes write only afterwards
-    {
-      static_assert((int64_t)kZScratchSlots * wide_z_slots<N, WW>() * N * WW <= (int64_t)N * N * half_pitch<N>(),
-                    "scratch exceeds Gy");
-      const size_t smem = wide_z_smem<N, WW>();
-      if ((rc = set_smem(k_fft_z_green_wide<N, WW>, smem))) return rc;
-      LaunchScope ls_(flabel<N>(1), st);
-      k_fft_z_green_wide<N, WW><<<grid, NT, smem, st>>>(A, Gz, Gy, kf, deconv, norm, tw, err);
-      COLA_LAUNCH_CHECK();
-    }
-  } else {
-    // 3. z pass with the Green's function
-    {
-      const size_t smem = sizeof(float2) * 2 * N * W;
-      if ((rc = set_smem(k_fft_z_green<N>, smem))) return rc;
-      dim3 grid((nh + W - 1) / W, N);
-      LaunchScope ls_(flabel<N>(1), st);
-      k_fft_z_green<N><<<grid, FFTConf<N>::T * W, smem, st>>>(A, Gz, P, kf, deconv, norm, tw);
-      COLA_LAUNCH_CHECK();
-    }
+  // 2. forward y pass
+  if ((rc = launch_fft_cols(N, false, A, N, (int64_t)N * P, P, nh, tw, st))) return rc;
+  constexpr int SL = cols_slabs<N>();
+  const dim3 grid((nh + W - 1) / W, N / SL);
+  // 3. z pass with the Green's function
+  {
+    constexpr size_t smem = z_smem<N>();
+    if ((rc = set_smem(k_fft_z_green<N>, smem))) return rc;
+    LaunchScope ls_(flabel<N>(1), st);
+    k_fft_z_green<N><<<grid, cols_threads<N>(), smem, st>>>(A, Gz, kf, deconv, norm, tw);
+    COLA_LAUNCH_CHECK();
   }
   // 4. inverse y passes
-  if constexpr (WI > 0) {
-    const dim3 grid((nh + WI - 1) / WI, N);
-    const size_t smem = sizeof(float2) * (N * WI + stw_size<FFTConf<N>>());
-    if ((rc = set_smem(k_fft_y_inv3_wide<N, WI>, smem))) return rc;
-    LaunchScope ls_(flabel<N>(2), st);
-    k_fft_y_inv3_wide<N, WI><<<grid, FFTConf<N>::T * WI, smem, st>>>(A, Gy, Gz, kf, tw);
-    COLA_LAUNCH_CHECK();
-  } else {
-    const size_t smem = sizeof(float2) * 2 * N * W;
+  {
+    constexpr size_t smem = sizeof(float2) * (SL * N * W + stw_size<FFTConf<N>>());
     if ((rc = set_smem(k_fft_y_inv3<N>, smem))) return rc;
-    dim3 grid((nh + W - 1) / W, N);
     LaunchScope ls_(flabel<N>(2), st);
-    k_fft_y_inv3<N><<<grid, FFTConf<N>::T * W, smem, st>>>(A, Gy, Gz, P, kf, tw);
+    k_fft_y_inv3<N><<<grid, cols_threads<N>(), smem, st>>>(A, Gy, Gz, kf, tw);
     COLA_LAUNCH_CHECK();
   }
   // 5. inverse x passes (persistent, bulk-copy pipelined)
@@ -356,7 +257,7 @@ int launch_density_spectrum(const Geometry& g, const Tiles& tl, const uint4* rec
   case N: {                                                                                           \
     int rc;                                                                                           \
     if ((rc = deposit_fftx_t<N>(g, tl, rec, offsets, A, P, tw, err, st))) return rc;                  \
-    if ((rc = forward_y_t<N>(A, P, tw, st))) return rc;                                               \
+    if ((rc = launch_fft_cols(N, false, A, N, (int64_t)N * P, P, N / 2 + 1, tw, st))) return rc;      \
     return launch_fft_cols(N, false, A, N, P, (int64_t)N * P, N / 2 + 1, tw, st); /* z: slab = y */ \
   }
     X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768) X(1024) X(1536) X(2048)
