@@ -446,8 +446,6 @@ int cola_status(cola_plan* plan, cola_stream stream) {
   COLA_CUDA_CHECK(cudaMemset(plan->ws.err, 0, sizeof(int)));
   if (err & kErrTimeout) return fail(COLA_ETIMEOUT, "a kernel gave up waiting for its bulk copies");
   if (err & kErrUnion) return fail(COLA_ETIMEOUT, "friends-of-friends: union-find retries ran out");
-  if (err & kErrSmIds)
-    return fail(COLA_EUNSUPPORTED, "the wide z pass found no scratch slot for its SM (more SM ids than slots)");
   if (err & kErrNonFinite) return fail(COLA_EOVERFLOW, "non-finite particle displacement");
   if (err & kErrOverflow) return fail(COLA_EOVERFLOW, "fixed-point density overflow (too many particles per cell)");
   return COLA_OK;

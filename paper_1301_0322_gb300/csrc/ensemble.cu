@@ -200,14 +200,21 @@ __global__ void __launch_bounds__(NT, 512 / NT) ke_cols(const BoxDesc* __restric
     using C = FFTConfV<N, V>;                                                                             \
     constexpr int W = NT / C::T, nbx = (N / 2 + 1 + W - 1) / W;                                           \
     const int bx = local % nbx, slab = local / nbx;                                                       \
+    const ColsGroup<N, W, float2, C> mem(sm, threadIdx.x, 0);                                             \
+    float2* stab = sm + N * W;                                                                            \
+    stw_fill<C, 1>(stab, d.tw, threadIdx.x, NT);                                                          \
+    const SmemTw<C> stw{stab};                                                                            \
+    const int64_t ystep = d.P, zstep = (int64_t)N * d.P;                                                  \
+    const StripWalk<N, W, float2, C> s(KIND == 1 ? ystep : zstep, KIND == 1 ? zstep : ystep, bx, slab, mem); \
+    const auto none = [] {};                                                                              \
     if constexpr (KIND == 0) {                                                                            \
-      float2* stab = sm + N * W;                                                                          \
-      stw_fill<C, 1>(stab, d.tw, threadIdx.x, NT);                                                        \
-      cols_body<N, W, 1, false, float2, C>(d.A, (int64_t)N * d.P, d.P, N / 2 + 1, SmemTw<C>{stab}, bx, slab, sm);    \
+      cols_strip<false>(d.A, s, stw, mem, none);                                                    \
     } else if constexpr (KIND == 1) {                                                                     \
-      z_green_body<N, W, 1, float2, C>(d.A, d.Gz, d.kf, d.deconv, d.norm, d.tw, bx, slab, sm, park);      \
+      float* sinc2 = reinterpret_cast<float*>(stab + stw_size<C>());                                      \
+      sinc2_fill<N>(sinc2, threadIdx.x, NT);                                                              \
+      z_green_strip(d.A, d.Gz, d.kf, d.deconv, d.norm, stw, sinc2, s, mem, park, none);                  \
     } else {                                                                                              \
-      y_inv3_body<N, W, 1, float2, C>(d.A, d.Gy, d.Gz, d.kf, d.tw, bx, slab, sm, park);                   \
+      y_inv3_strip(d.A, d.Gy, d.Gz, d.kf, stw, s, mem, park, none);                                      \
     }                                                                                                     \
   } break;
       COLA_ENS_SIZES(X)
@@ -616,7 +623,7 @@ int configure(cola_ensemble* e, cudaStream_t st) {
     c2r_buf = std::max(c2r_buf, (size_t)sh.RB * xrow_ld_host(M));
     e->smem[kKDeposit] = std::max(e->smem[kKDeposit], dep);
     e->smem[kKYfwd] = std::max(e->smem[kKYfwd], cols);
-    e->smem[kKZgreen] = std::max(e->smem[kKZgreen], cols + sizeof(float2) * ((n + sh.W + 3) / 4 * 2));
+    e->smem[kKZgreen] = std::max(e->smem[kKZgreen], cols + sizeof(float) * n);
     e->smem[kKYinv] = std::max(e->smem[kKYinv], cols);
   }
   if (bins > e->max_bins_total) return fail(COLA_EINVAL, "ensemble: bin count above the workspace sizing");

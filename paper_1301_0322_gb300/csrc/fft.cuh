@@ -374,6 +374,29 @@ struct SmemTw {
 };
 
 // ---- Stockham stages --------------------------------------------------------------------
+// exchange slot base + off, where off is a constant once the loops are unrolled and the two share
+// no bit below 16: the buffer's own at(base, off) where it has one (a permuted layout)
+template <class Mem, class = void>
+struct HasAt : std::false_type {};
+template <class Mem>
+struct HasAt<Mem, std::void_t<decltype(std::declval<const Mem&>().at(0, 0))>> : std::true_type {};
+template <class Mem>
+__device__ __forceinline__ decltype(auto) mem_at(Mem& mem, int base, int off) {
+  if constexpr (HasAt<Mem>::value) return mem.at(base, off);
+  else return mem(base + off);
+}
+// barrier of the threads that share an exchange buffer: the buffer's own sync() where it has one
+// (a part of the block), else the block's
+template <class Mem, class = void>
+struct HasSync : std::false_type {};
+template <class Mem>
+struct HasSync<Mem, std::void_t<decltype(std::declval<const Mem&>().sync())>> : std::true_type {};
+template <class Mem>
+__device__ __forceinline__ void stage_sync(const Mem& mem) {
+  if constexpr (HasSync<Mem>::value) mem.sync();
+  else __syncthreads();
+}
+
 template <int N, int E, int TWS, bool INV>
 struct Stockham {
   static constexpr int T = N / E;
@@ -426,6 +449,36 @@ struct Stockham {
     }
   }
 
+  // out_index as a part that depends on the thread and one that does not (constant after unrolling)
+  template <int R, int NS>
+  __device__ __forceinline__ static int out_base(int t) {
+    if constexpr (T % NS == 0) return (int)(((unsigned)t / NS) * (NS * R) + (unsigned)t % NS);
+    else return t;
+  }
+  template <int R, int NS>
+  __device__ __forceinline__ static constexpr int out_off(int q, int r) {
+    if constexpr (T % NS == 0) return q * (T * R) + r * NS;
+    else return T * q + r * NS;
+  }
+  // exchange after the stage (R, NS): this thread's outputs to the buffer, the next stage's inputs from it
+  template <int R, int NS, int R2, class V, class Mem>
+  __device__ __forceinline__ static void exchange(V (&v)[E], int t, Mem& mem) {
+    constexpr bool split = T % NS == 0 || NS >= T * (E / R);
+    const int base = split ? out_base<R, NS>(t) : 0;
+#pragma unroll
+    for (int q = 0; q < E / R; ++q)
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if constexpr (split) mem_at(mem, base, out_off<R, NS>(q, r)) = v[q * R + r];
+        else mem_at(mem, out_index<R, NS>(t, q, r), 0) = v[q * R + r];
+      }
+    stage_sync(mem);
+#pragma unroll
+    for (int q = 0; q < E / R2; ++q)
+#pragma unroll
+      for (int r = 0; r < R2; ++r) v[q * R2 + r] = mem_at(mem, t, T * q + r * (N / R2));
+  }
+
   // Run the stages NS.. of the radix list.  v holds the inputs of the first listed stage.
   // mem(n) -> V& : exchange buffer slot for element n of this thread's sequence.
   // store(n, x)       : final output of element n.
@@ -439,7 +492,7 @@ struct Stockham {
     if constexpr (sizeof...(Rest) == 0) {
       static_assert(NS * R == N, "radix list does not multiply to N");
       if constexpr (NS == 1) before();
-      __syncthreads();
+      stage_sync(mem);
       if constexpr (NS == 1) after();
 #pragma unroll
       for (int q = 0; q < E / R; ++q)
@@ -447,46 +500,31 @@ struct Stockham {
         for (int r = 0; r < R; ++r) store(out_index<R, NS>(t, q, r), v[q * R + r]);
     } else {
       if constexpr (NS == 1) before();
-      __syncthreads();
+      stage_sync(mem);
       if constexpr (NS == 1) after();
-#pragma unroll
-      for (int q = 0; q < E / R; ++q)
-#pragma unroll
-        for (int r = 0; r < R; ++r) mem(out_index<R, NS>(t, q, r)) = v[q * R + r];
-      __syncthreads();
-      constexpr int R2 = FirstRadix<Radices<Rest...>>::value;
-#pragma unroll
-      for (int q = 0; q < E / R2; ++q)
-#pragma unroll
-        for (int r = 0; r < R2; ++r) v[q * R2 + r] = mem(t + T * q + r * (N / R2));
+      exchange<R, NS, FirstRadix<Radices<Rest...>>::value>(v, t, mem);
       run<NS * R, Rest...>(v, t, tw, mem, store, before, after);
     }
   }
 
-  // The stages NS.. with the result left in registers, in the last stage's order.
-  template <int NS, int R, int... Rest, class V, class TW, class Mem>
-  __device__ __forceinline__ static void run_regs(V (&v)[E], int t, const TW& tw, Mem& mem) {
+  // The stages NS.. with the result left in registers, in the last stage's order.  after_reads()
+  // is called once this thread has read its inputs of the last stage.
+  template <int NS, int R, int... Rest, class V, class TW, class Mem, class Hook>
+  __device__ __forceinline__ static void run_regs(V (&v)[E], int t, const TW& tw, Mem& mem, Hook& after_reads) {
     compute<R, NS>(v, t, tw);
     if constexpr (sizeof...(Rest) > 0) {
-      __syncthreads();
-#pragma unroll
-      for (int q = 0; q < E / R; ++q)
-#pragma unroll
-        for (int r = 0; r < R; ++r) mem(out_index<R, NS>(t, q, r)) = v[q * R + r];
-      __syncthreads();
-      constexpr int R2 = FirstRadix<Radices<Rest...>>::value;
-#pragma unroll
-      for (int q = 0; q < E / R2; ++q)
-#pragma unroll
-        for (int r = 0; r < R2; ++r) v[q * R2 + r] = mem(t + T * q + r * (N / R2));
-      run_regs<NS * R, Rest...>(v, t, tw, mem);
+      stage_sync(mem);
+      exchange<R, NS, FirstRadix<Radices<Rest...>>::value>(v, t, mem);
+      if constexpr (sizeof...(Rest) == 1) after_reads();
+      run_regs<NS * R, Rest...>(v, t, tw, mem, after_reads);
     } else {
-      static_assert(NS * R == N, "radix list does not multiply to N");
+      static_assert(NS * R == N && NS > 1, "radix list of at least two stages that multiplies to N");
     }
   }
-  template <int... Rs, class V, class TW, class Mem>
-  __device__ __forceinline__ static void run_regs_all(Radices<Rs...>, V (&v)[E], int t, const TW& tw, Mem& mem) {
-    run_regs<1, Rs...>(v, t, tw, mem);
+  template <int... Rs, class V, class TW, class Mem, class Hook>
+  __device__ __forceinline__ static void run_regs_all(Radices<Rs...>, V (&v)[E], int t, const TW& tw, Mem& mem,
+                                                      Hook& after_reads) {
+    run_regs<1, Rs...>(v, t, tw, mem, after_reads);
   }
 
   template <int... Rs, class V, class TW, class Mem, class Store, class Before, class After>
@@ -523,8 +561,9 @@ __device__ __forceinline__ void fft_1d(int t, const TW& tw, Load& load, Mem& mem
 // Both the first stage's inputs and the last stage's outputs of a thread are the elements
 // congruent to t modulo T, so a thread can go from one transform to the next without an exchange.
 // (The first exchange starts with a block barrier; none follows the last one's reads.)
-template <int N, int TWS, bool INV, class C = FFTConf<N>, class V, class TW, class Mem>
-__device__ __forceinline__ void fft_regs(V (&u)[C::E], int t, const TW& tw, Mem& mem) {
+// after_reads() runs when this thread has read the last stage's inputs.
+template <int N, int TWS, bool INV, class C = FFTConf<N>, class V, class TW, class Mem, class Hook>
+__device__ __forceinline__ void fft_regs(V (&u)[C::E], int t, const TW& tw, Mem& mem, Hook& after_reads) {
   static_assert(C::N == N, "configuration of another length");
   constexpr int E = C::E;
   constexpr int R0 = FirstRadix<typename C::radices>::value, RL = last_radix_of(typename C::radices{});
@@ -533,11 +572,16 @@ __device__ __forceinline__ void fft_regs(V (&u)[C::E], int t, const TW& tw, Mem&
   for (int q = 0; q < E / R0; ++q)
 #pragma unroll
     for (int r = 0; r < R0; ++r) v[q * R0 + r] = u[q + r * (E / R0)];
-  Stockham<N, E, TWS, INV>::run_regs_all(typename C::radices{}, v, t, tw, mem);
+  Stockham<N, E, TWS, INV>::run_regs_all(typename C::radices{}, v, t, tw, mem, after_reads);
 #pragma unroll
   for (int q = 0; q < E / RL; ++q)
 #pragma unroll
     for (int r = 0; r < RL; ++r) u[q + r * (E / RL)] = v[q * RL + r];
+}
+template <int N, int TWS, bool INV, class C = FFTConf<N>, class V, class TW, class Mem>
+__device__ __forceinline__ void fft_regs(V (&u)[C::E], int t, const TW& tw, Mem& mem) {
+  auto none = [] {};
+  fft_regs<N, TWS, INV, C>(u, t, tw, mem, none);
 }
 
 }  // namespace cola

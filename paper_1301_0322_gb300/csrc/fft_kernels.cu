@@ -6,6 +6,7 @@
 #include "cola_internal.cuh"
 #include "fft.cuh"
 #include "pm_bodies.cuh"
+#include "cols_launch.cuh"
 
 namespace cola {
 
@@ -15,18 +16,19 @@ __host__ __device__ constexpr int x_rows() {
   return FFTConf<N / 2>::T >= 256 ? 1 : 256 / FFTConf<N / 2>::T;
 }
 
-// In-place FFT of ncols columns per slab: element (n, col) at data[slab*slab_stride + n*row_stride + col].
-// Strips of cols_width columns, two per thread; stage twiddles from shared memory.
+// In-place FFT of the N/2 + 1 columns of nslabs slabs: element (n, col) at data[slab*slab_stride + n*row_stride + col].
 template <int N, bool INV>
-__global__ void __launch_bounds__(cols_threads<N>(), cols_min_blocks<N>())
-    k_fft_cols(float2* __restrict__ data, int64_t slab_stride, int64_t row_stride, int ncols,
+__global__ void __launch_bounds__(ColsCfg<N, kColsPlain>::THREADS, ColsCfg<N, kColsPlain>::MIN_BLOCKS)
+    k_fft_cols(float2* __restrict__ data, int64_t slab_stride, int64_t row_stride, int nslabs,
                const float2* __restrict__ tw) {
   extern __shared__ __align__(16) float2 smem[];
-  constexpr int W = cols_width<N>(), SL = cols_slabs<N>();
-  float2* stab = smem + SL * N * W;
-  stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, cols_threads<N>());
-  cols_body<N, W, SL, INV, cpair>(data, slab_stride, row_stride, ncols, SmemTw<FFTConf<N>>{stab}, blockIdx.x,
-                                  blockIdx.y * SL, smem);
+  using Cfg = ColsCfg<N, kColsPlain>;
+  float2* stab = smem + Cfg::TABLE;
+  stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
+  __syncthreads();
+  const SmemTw<FFTConf<N>> stw{stab};
+  cols_walk<Cfg>(data, slab_stride, row_stride, nslabs, smem,
+                 [&](const auto& s, const auto& mem, auto& next) { cols_strip<INV>(data, s, stw, mem, next); });
 }
 
 // Real rows of length N -> half-spectrum rows (N/2 + 1 entries, stride P), via a complex
@@ -137,18 +139,20 @@ static int x_c2r(const float2* in, float* out, int64_t nrows, int P, const float
 template <int N>
 static int cols(bool inverse, float2* data, int64_t nslabs, int64_t slab_stride, int64_t row_stride, int ncols,
                 const float2* tw, cudaStream_t st) {
-  constexpr int W = cols_width<N>(), SL = cols_slabs<N>();
-  const size_t smem = (size_t)(SL * N * W + stw_size<FFTConf<N>>()) * sizeof(float2);
-  if (nslabs > 65535 || nslabs % SL) return fail(COLA_EINVAL, "fft column pass: unexpected number of slabs");
-  dim3 grid((ncols + W - 1) / W, (unsigned)(nslabs / SL));
+  if (nslabs > 65535 || ncols != N / 2 + 1) return fail(COLA_EINVAL, "fft column pass: unexpected slabs or columns");
+  using Cfg = ColsCfg<N, kColsPlain>;
+  const int64_t strips = Cfg::STRIPS * nslabs;
+  constexpr size_t smem = cols_smem<Cfg>(0);
+  unsigned grid = 0;
+  int rc;
   if (inverse) {
-    allow_smem(k_fft_cols<N, true>, smem);
-    { LaunchScope ls_(label<N>("inv"), st);
-    k_fft_cols<N, true><<<grid, cols_threads<N>(), smem, st>>>(data, slab_stride, row_stride, ncols, tw); }
+    if ((rc = cols_grid<Cfg, k_fft_cols<N, true>>(smem, strips, &grid))) return rc;
+    LaunchScope ls_(label<N>("inv"), st);
+    k_fft_cols<N, true><<<grid, Cfg::THREADS, smem, st>>>(data, slab_stride, row_stride, (int)nslabs, tw);
   } else {
-    allow_smem(k_fft_cols<N, false>, smem);
-    { LaunchScope ls_(label<N>("fwd"), st);
-    k_fft_cols<N, false><<<grid, cols_threads<N>(), smem, st>>>(data, slab_stride, row_stride, ncols, tw); }
+    if ((rc = cols_grid<Cfg, k_fft_cols<N, false>>(smem, strips, &grid))) return rc;
+    LaunchScope ls_(label<N>("fwd"), st);
+    k_fft_cols<N, false><<<grid, Cfg::THREADS, smem, st>>>(data, slab_stride, row_stride, (int)nslabs, tw);
   }
   COLA_LAUNCH_CHECK();
   return COLA_OK;

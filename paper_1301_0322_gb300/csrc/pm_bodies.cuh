@@ -63,32 +63,64 @@ __host__ __device__ constexpr int half_pitch() {
   return ((N / 2 + 1) + 3) / 4 * 4;
 }
 
-// Strip width (columns per block), slabs per block, threads and resident blocks per SM of the
-// single-box column passes, two columns per thread: 16 columns are 128-byte row segments, 8 where
-// a strip of 16 would leave room for fewer than two blocks in shared memory.  The registers of E
-// complex pairs (4 E) set the threads per SM.
-template <int N>
-__host__ __device__ constexpr int cols_width() {
-  return N >= 512 ? 8 : 16;
-}
-// two slabs per block where one makes a block of one or two warps whose parked words take a
-// quarter of the tensor memory
-template <int N>
-__host__ __device__ constexpr int cols_slabs() {
-  return N == 192 || N == 96 ? 2 : 1;
-}
-template <int N>
-__host__ __device__ constexpr int cols_threads() {
-  return FFTConf<N>::T * cols_width<N>() / 2 * cols_slabs<N>();
-}
-template <int N>
-__host__ __device__ constexpr int cols_min_blocks() {
-  constexpr int E = FFTConf<N>::E, threads = cols_threads<N>();
-  constexpr int per_sm = (E >= 24 ? 384 : (E >= 12 ? 512 : 768)) / threads;
-  // (and no more blocks than have their parked words in the tensor memory at once)
-  constexpr int parked = 512 / tmem_columns(threads, (4 * E + 15) / 16 * 16);
-  return per_sm < 1 ? 1 : (per_sm < parked ? per_sm : parked);
-}
+// Shapes of the single-box column passes.  A block holds G groups of threads, each with an
+// exchange buffer and a barrier of its own, which transform strips of W columns independently of
+// one another (one group's loads and stores overlap another's transforms) and share the stage
+// twiddle table.
+//
+// What bounds them: shared-memory wavefronts (each exchange writes and reads every element) and
+// how many bytes they keep in flight.  Loads go through the asynchronous copies of copy_async16
+// into the exchange buffer itself: through the L1 cache each 64-byte row segment held a 128-byte
+// line until it returned, and a kernel that takes 200 KB of shared memory has few lines left.
+// More strips in flight than the shapes below have were slower (768: forward y 659 us with two
+// strips of 8 columns per SM, 747 with three, 1080 with four), as were the E complex pairs of a
+// thread squeezed into fewer registers; wider strips move more of a DRAM page at once (1024: z
+// 4987 us with strips of 8, 4190 with 16).  Event times in us per launch, one column per thread
+// with two-pass or re-read strips -> these shapes (GB300):
+//   mesh   forward y       z with Green's function   inverse y
+//    256    24 ->   26        68 ->    57               68 ->    64
+//    384    95 ->   84       271 ->   195              303 ->   220
+//    512   246 ->  198       953 ->   448             1172 ->   550
+//    768   734 ->  655      2222 ->  1660             2133 ->  1880
+//   1024  1922 -> 1714      8445 ->  4190             9090 ->  4710
+//   1536  7657 -> 6030     29898 -> 19700            24573 -> 18600
+enum ColsKind { kColsPlain, kColsZ, kColsY };
+template <int N, int W, class V, class C>
+struct ColsGroup;
+template <int N, int KIND>
+struct ColsCfg {
+  using C = FFTConf<N>;
+  static constexpr int N_ = N;
+  // two columns per thread from 256 up; below, one, on twice the threads
+  using V = std::conditional_t<(N >= 256), cpair, float2>;
+  // 16 columns are 128-byte row segments; 8 where buffers of 16 do not fit
+  static constexpr int W = (N >= 1536 || (N == 768 && KIND == kColsY)) ? 8 : 16;
+  // groups per block
+  static constexpr int G = N == 1536 && KIND == kColsPlain ? 2
+                           : N == 768                      ? (KIND == kColsPlain ? 1 : 2)
+                           : N == 512                      ? 2
+                           : N == 384                      ? (KIND == kColsPlain ? 2 : 3)
+                                                           : 1;
+  // threads per SM the kernel is compiled for (its registers)
+  static constexpr int PER_SM = N == 2048   ? 512
+                                : N == 1536 ? (KIND == kColsPlain ? 512 : 256)
+                                : N == 1024 ? 512
+                                : N == 768  ? (KIND == kColsZ ? 512 : 256)
+                                : N == 512  ? 1024
+                                : N == 384  ? (KIND == kColsPlain ? 256 : 384)
+                                            : 512;
+  // persistent blocks, one wave of them, from 384 up
+  static constexpr bool RESIDENT = N >= 384;
+  static constexpr int K = lanes_of<V>(), GROUP = C::T * W / K, THREADS = GROUP * G;
+  static constexpr int WORDS = (2 * C::E * K + 15) / 16 * 16;  // parked words per thread
+  // (no more blocks than have their parked words in the tensor memory at once)
+  static constexpr int PARKED = KIND == kColsPlain ? 64 : 512 / tmem_columns(THREADS, WORDS);
+  static constexpr int WANT = PER_SM / THREADS < 1 ? 1 : PER_SM / THREADS;
+  static constexpr int MIN_BLOCKS = WANT < PARKED ? WANT : PARKED;
+  static constexpr int STRIPS = (N / 2 + W) / W;  // per slab
+  static constexpr int TABLE = G * N * W;         // float2 offset of the stage twiddle table
+  using Group = ColsGroup<N, W, V, C>;
+};
 // one thread's E elements, parked (tmem.cuh)
 template <int THREADS, int E, class V>
 using Park = TmemPark<THREADS, (E * lanes_of<V>() * 2 + 15) / 16 * 16>;
@@ -123,38 +155,133 @@ __device__ __forceinline__ void park_load(const P& park, V (&u)[E]) {
   }
 }
 
-// This thread's place in a block that takes W columns of each of SL slabs: columns w K .. of the
-// strip, transform thread t, slab number sub; strips of the exchange buffer slab after slab.
-template <int N, int W, int SL, class V, class C>
-struct ColsThread {
-  static constexpr int K = lanes_of<V>(), WT = W / K, T = C::T, NT = T * WT * SL;
-  int w, t, sub;
+// A thread's place in a group that transforms a strip of W columns, and the group's exchange
+// buffer: columns w K .. of the strip, transform thread t.  Rows of 64 bytes (W = 8) are swapped
+// in pairs according to the parity of n / R0, so that the first stage's stores, which are R0 rows
+// apart in consecutive threads, do not all fall on the same half of the banks.
+template <int N, int W, class V, class C>
+struct ColsGroup {
+  static constexpr int K = lanes_of<V>(), WT = W / K, T = C::T, NT = T * WT;
+  // (the exponent of R0; 0 = rows in place, also where T would not keep the loads' parity constant)
+  static constexpr int SHIFT = first_radix<C>() >= 16 ? 4 : 3;
+  static constexpr int SWAP = W * (int)sizeof(float2) == 64 && T % (2 << SHIFT) == 0 ? SHIFT : 0;
+  int w, t, bar;
   V* S;
-  __device__ __forceinline__ explicit ColsThread(float2* smem) {
-    const int i = threadIdx.x;
-    w = i % WT;
-    t = i / WT % T;
-    sub = SL == 1 ? 0 : i / (WT * T);
-    S = reinterpret_cast<V*>(smem) + (SL == 1 ? 0 : sub * (N * WT));
+  // thread i of the group, its buffer of N W float2 and its hardware barrier
+  __device__ __forceinline__ ColsGroup(float2* buf, int i, int barrier)
+      : w(i % WT), t(i / WT), bar(barrier), S(reinterpret_cast<V*>(buf)) {}
+  // row n = base + off (see mem_at): n ^ ((n >> SWAP) & 1), of which base gives two values (in
+  // registers) and off the choice between them and a constant offset
+  __device__ __forceinline__ V& at(int base, int off) const {
+    if constexpr (SWAP > 0) {
+      const int x = base ^ ((base >> SWAP) & 1);
+      return (((off ^ (off >> SWAP)) & 1) ? S + ((x ^ 1) * WT + w) : S + (x * WT + w))[(off & ~1) * WT];
+    } else {
+      return (S + (base * WT + w))[off * WT];
+    }
   }
-  __device__ __forceinline__ V& operator()(int n) const { return S[n * WT + w]; }
+  // The same place with its indices recomputed from here on: keeps a persistent loop from holding
+  // every address of the exchange in a register (at 128 registers those would be spilled).
+  __device__ __forceinline__ ColsGroup fresh() const {
+    ColsGroup g = *this;
+    asm volatile("" : "+r"(g.w), "+r"(g.t));
+    return g;
+  }
+  __device__ __forceinline__ void sync() const {
+    if constexpr (NT == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory");
+  }
+  // Start the copies of this thread's elements n = t + T m (at p + m step) into their slots of the
+  // buffer; collect() waits for them.  No other thread touches those slots before the first
+  // exchange, and the caller sees to it that the group has read the buffer's last contents.
+  // (Scalar columns are 8 bytes wide: they are loaded by collect() itself.)
+  __device__ __forceinline__ void fetch(const float2* p, int64_t step, bool valid) const {
+    if constexpr (K == 2) {
+#pragma unroll
+      for (int m = 0; m < C::E; ++m, p += step) copy_async16(&at(t, T * m), p, valid);
+    }
+  }
+  __device__ __forceinline__ void collect(V (&u)[C::E], const float2* p, int64_t step, bool valid) const {
+    if constexpr (K == 2) {
+      copy_wait_all();
+#pragma unroll
+      for (int m = 0; m < C::E; ++m) {
+        const V& slot = at(t, T * m);
+        u[m] = c_interleave(*reinterpret_cast<const float4*>(&slot));
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < C::E; ++m, p += step) u[m] = valid ? c_load<V>(p) : c_zero<V>();
+    }
+  }
 };
 
-// block (bx, slab0): W columns of SL slabs of the in-place strided FFT (T(N) * W / lanes * SL
-// threads); smem: SL N W float2.  Element (n, col) at data[slab * slab_stride + n * row_stride + col].
-// (tw: the base twiddle table or an SmemTw stage table)
-template <int N, int W, int SL, bool INV, class V, class C = FFTConf<N>, class TW>
-__device__ __forceinline__ void cols_body(float2* __restrict__ data, int64_t slab_stride, int64_t row_stride,
-                                          int ncols, const TW& tw, int bx, int slab0, float2* smem) {
-  const ColsThread<N, W, SL, V, C> mem(smem);
-  const int col = bx * W + mem.w * mem.K;
-  const bool valid = col < ncols;
-  float2* base = data + (int64_t)(slab0 + mem.sub) * slab_stride + (valid ? col : 0);
-  auto load = [&](int n) -> V { return valid ? c_load<V>(base + (int64_t)n * row_stride) : c_zero<V>(); };
-  auto store = [&](int n, V x) {
-    if (valid) c_store(base + (int64_t)n * row_stride, x);
+// The strips of one column pass: strip i covers W columns from bx W of one slab (i = slab NB + bx,
+// NB strips per slab); element (n, col) of it at data[slab * slab_stride + n * row_stride + col].
+// A thread's first element of strip i, and whether its columns exist:
+template <int N, int W, class V, class C>
+struct StripWalk {
+  int64_t slab_stride, row_stride;
+  int kx, slab;
+  bool valid;
+  int64_t first;
+  __device__ __forceinline__ StripWalk(int64_t slab_stride_, int64_t row_stride_, int bx, int slab_,
+                                       const ColsGroup<N, W, V, C>& g)
+      : slab_stride(slab_stride_), row_stride(row_stride_), kx(bx * W + g.w * g.K), slab(slab_), valid(kx < N / 2 + 1),
+        first(slab * slab_stride + g.t * row_stride + (valid ? kx : 0)) {}
+  __device__ __forceinline__ int64_t step() const { return C::T * row_stride; }
+};
+
+// In-place FFT of a strip whose copies are under way; next() starts those of the group's next
+// strip, once the group is done with the buffer and before the last stage and the stores.
+template <bool INV, int N, int W, class V, class C, class TW, class Next>
+__device__ __forceinline__ void cols_strip(float2* __restrict__ data, const StripWalk<N, W, V, C>& s, const TW& tw,
+                                           const ColsGroup<N, W, V, C>& mem, Next&& next) {
+  constexpr int E = C::E;
+  float2* p = data + s.first;
+  V u[E];
+  mem.collect(u, p, s.step(), s.valid);
+  auto after_reads = [&] {
+    mem.sync();
+    next();
   };
-  fft_1d<N, 1, INV, C>(mem.t, tw, load, mem, store);
+  fft_regs<N, 1, INV, C>(u, mem.t, tw, mem, after_reads);
+  if (s.valid) {
+#pragma unroll
+    for (int m = 0; m < E; ++m, p += s.step()) c_store(p, u[m]);
+  }
+}
+
+// The walk of a group over the strips of nslabs slabs (the blocks' first groups take the first
+// strips, then the second groups, ...): one(walk, mem, next) transforms a strip whose copies from
+// src are under way and calls next() where its buffer is free for the following strip's.
+template <class Cfg, class One>
+__device__ __forceinline__ void cols_walk(const float2* src, int64_t slab_stride, int64_t row_stride, int nslabs,
+                                          float2* smem, One&& one) {
+  constexpr int G = Cfg::G, NB = Cfg::STRIPS, N = Cfg::N_;
+  static_assert(G <= 15, "hardware barriers: 0 is the block's, 1 to 15 the groups'");
+  using Group = typename Cfg::Group;
+  using Walk = StripWalk<N, Cfg::W, typename Cfg::V, typename Cfg::C>;
+  const int group = threadIdx.x / Cfg::GROUP;
+  const Group place(smem + group * (N * Cfg::W), threadIdx.x % Cfg::GROUP, group + 1);
+  const int total = NB * nslabs, stride = gridDim.x * G;
+  int i = blockIdx.x + gridDim.x * group;
+  if (i < total) {
+    const Walk s(slab_stride, row_stride, i % NB, i / NB, place);
+    place.fetch(src + s.first, s.step(), s.valid);
+  }
+  for (; i < total; i += stride) {
+    const Group mem = place.fresh();
+    const Walk s(slab_stride, row_stride, i % NB, i / NB, mem);
+    auto next = [&] {
+      const int j = i + stride;
+      if (j < total) {
+        const Walk n(slab_stride, row_stride, j % NB, j / NB, mem);
+        mem.fetch(src + n.first, n.step(), n.valid);
+      }
+    };
+    one(s, mem, next);
+  }
 }
 
 // ---- 1. deposit + x r2c -----------------------------------------------------------------------
@@ -291,13 +418,6 @@ __device__ __forceinline__ void deposit_fftx_body(const Geometry& g, const Tiles
 // thread ends a transform with the elements the next one starts from, so phi stays in its
 // registers and its second use is parked in tensor memory.
 //
-// shared-memory layout: SL strips (N W float2 each), sinc^2 tables (N + W floats, rounded up to
-// 16 bytes), stage twiddle table
-template <int N, int W, int SL>
-__host__ __device__ constexpr int z_table_offset() {
-  return SL * N * W + (N + W + 3) / 4 * 2;
-}
-
 // norm / (kf2 m2 W^p): the Green's function of one mode (wk = W(k))
 __device__ __forceinline__ float green_of(int m2, float kf2, float wk, int deconv, float norm) {
   float gk = 0.0f;
@@ -309,48 +429,44 @@ __device__ __forceinline__ float green_of(int m2, float kf2, float wk, int decon
   return gk;
 }
 
-// block (bx, ky0): W columns kx of SL slabs ky (T(N) W / lanes SL threads)
-template <int N, int W, int SL, class V, class C = FFTConf<N>, class P_>
-__device__ __forceinline__ void z_green_body(float2* __restrict__ A, float2* __restrict__ Gz, float kf, int deconv,
-                                             float norm, const float2* __restrict__ tw, int bx, int ky0, float2* sm,
-                                             const P_& park) {
-  constexpr int K = lanes_of<V>(), E = C::E, T = C::T, nh = N / 2 + 1, P = half_pitch<N>();
-  const ColsThread<N, W, SL, V, C> mem(sm);
-  float* sz2 = reinterpret_cast<float*>(sm + SL * N * W);
-  float* sx2 = sz2 + N;
-  float2* stab = sm + z_table_offset<N, W, SL>();
-  stw_fill<C, 1>(stab, tw, threadIdx.x, mem.NT);
-  const SmemTw<C> stw{stab};
-  const int t = mem.t, ky = ky0 + mem.sub;
-  const int kx = bx * W + mem.w * K;
-  const bool valid = kx < nh;
-  constexpr int64_t zstride = (int64_t)N * P;
-  const int64_t at = (int64_t)ky * P + (valid ? kx : 0) + t * zstride;
-  float2* a = A + at;
-  float2* gz = Gz + at;
-  V u[E];
-#pragma unroll
-  for (int m = 0; m < E; ++m) u[m] = valid ? c_load<V>(a + m * (T * zstride)) : c_zero<V>();
-  for (int n = threadIdx.x; n < N + W; n += mem.NT) {
-    const float sv = n < N ? sinc_pi_f(signed_mode(n, N), N) : sinc_pi_f(bx * W + (n - N), N);
-    (n < N ? sz2[n] : sx2[n - N]) = sv * sv;
+// sinc^2 of the N mode numbers of a mesh side, into shared memory by threads tid of nth
+template <int N>
+__device__ __forceinline__ void sinc2_fill(float* dst, int tid, int nth) {
+  for (int n = tid; n < N; n += nth) {
+    const float sv = sinc_pi_f(signed_mode(n, N), N);
+    dst[n] = sv * sv;
   }
+}
+
+// one strip (slab = ky) whose copies are under way (sinc2: the table above; next: see cols_strip)
+template <int N, int W, class V, class C, class TW, class P_, class Next>
+__device__ __forceinline__ void z_green_strip(float2* __restrict__ A, float2* __restrict__ Gz, float kf, int deconv,
+                                              float norm, const TW& stw, const float* sinc2,
+                                              const StripWalk<N, W, V, C>& s, const ColsGroup<N, W, V, C>& mem,
+                                              const P_& park, Next&& next) {
+  constexpr int K = lanes_of<V>(), E = C::E, T = C::T;
+  constexpr int64_t zstep = (int64_t)T * N * half_pitch<N>();
+  const int t = mem.t, kx = s.kx;
+  float2* a = A + s.first;
+  float2* gz = Gz + s.first;
+  V u[E];
+  mem.collect(u, a, zstep, s.valid);
   fft_regs<N, 1, false, C>(u, t, stw, mem);
   {
-    const int ny = signed_mode(ky, N);
-    const float sy = sinc_pi_f(ny, N);
-    const float wy = sy * sy;
+    // (sinc is even: sinc2[k] is that of the mode numbers k and -k; the columns beyond N/2 are padding)
+    const int ny = signed_mode(s.slab, N);
+    const float wy = sinc2[s.slab];
     const float kf2 = kf * kf;
-    const float wxy0 = sx2[mem.w * K] * wy, wxy1 = sx2[mem.w * K + K - 1] * wy;
+    const float wxy0 = sinc2[s.valid ? kx : 0] * wy, wxy1 = sinc2[s.valid ? kx + K - 1 : 0] * wy;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
       const int n = t + T * m, nz = signed_mode(n, N);
       const int myz = ny * ny + nz * nz;
-      const float s0 = green_of(kx * kx + myz, kf2, wxy0 * sz2[n], deconv, norm);
+      const float s0 = green_of(kx * kx + myz, kf2, wxy0 * sinc2[n], deconv, norm);
       if constexpr (K == 1) {
         u[m] = c_scale(u[m], s0);
       } else {
-        const float s1 = green_of((kx + 1) * (kx + 1) + myz, kf2, wxy1 * sz2[n], deconv, norm);
+        const float s1 = green_of((kx + 1) * (kx + 1) + myz, kf2, wxy1 * sinc2[n], deconv, norm);
         u[m] = c_scale(u[m], make_float2(s0, s1));
       }
     }
@@ -362,49 +478,40 @@ __device__ __forceinline__ void z_green_body(float2* __restrict__ A, float2* __r
     u[m] = mul_ik(u[m], (n == N / 2) ? 0.0f : kf * (float)signed_mode(n, N));
   }
   fft_regs<N, 1, true, C>(u, t, stw, mem);
-  if (valid) {
+  if (s.valid) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) c_store(gz + m * (T * zstride), u[m]);
+    for (int m = 0; m < E; ++m) c_store(gz + m * zstep, u[m]);
   }
   __syncwarp();
   park_load(park, u);
-  fft_regs<N, 1, true, C>(u, t, stw, mem);
-  if (valid) {
+  auto after_reads = [&] {
+    mem.sync();
+    next();
+  };
+  fft_regs<N, 1, true, C>(u, t, stw, mem, after_reads);
+  if (s.valid) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) c_store(a + m * (T * zstride), u[m]);
+    for (int m = 0; m < E; ++m) c_store(a + m * zstep, u[m]);
   }
   __syncwarp();
 }
 
 // ---- 4. inverse y passes ------------------------------------------------------------------------------------
 // Gy = IFFT_y(i k_y B), then B = IFFT_y(B) in place, then Gz = IFFT_y(Gz): the strip of B is read
-// once and parked in tensor memory for its second transform.  block (bx, z0): W columns kx of SL
-// slabs z (T(N) W / lanes SL threads); sm: SL N W float2, then the stage twiddle table
-template <int N, int W, int SL, class V, class C = FFTConf<N>, class P_>
-__device__ __forceinline__ void y_inv3_body(float2* __restrict__ B, float2* __restrict__ Gy, float2* __restrict__ Gz,
-                                            float kf, const float2* __restrict__ tw, int bx, int z0, float2* sm,
-                                            const P_& park) {
-  constexpr int K = lanes_of<V>(), E = C::E, T = C::T, nh = N / 2 + 1, P = half_pitch<N>();
-  const ColsThread<N, W, SL, V, C> mem(sm);
-  float2* stab = sm + SL * N * W;
-  stw_fill<C, 1>(stab, tw, threadIdx.x, mem.NT);
-  const SmemTw<C> stw{stab};
+// once and parked in tensor memory for its second transform, after whose last exchange the copies
+// of the Gz strip start.  One strip (slab = z) whose copies of B are under way (next: see
+// cols_strip).
+template <int N, int W, class V, class C, class TW, class P_, class Next>
+__device__ __forceinline__ void y_inv3_strip(float2* __restrict__ B, float2* __restrict__ Gy, float2* __restrict__ Gz,
+                                             float kf, const TW& stw, const StripWalk<N, W, V, C>& s,
+                                             const ColsGroup<N, W, V, C>& mem, const P_& park, Next&& next) {
+  constexpr int E = C::E, T = C::T, step = T * half_pitch<N>();
   const int t = mem.t;
-  const int kx = bx * W + mem.w * K;
-  const bool valid = kx < nh;
-  const int64_t at = (int64_t)(z0 + mem.sub) * N * P + (valid ? kx : 0) + t * P;
-  float2* b = B + at;
-  float2* gy = Gy + at;
-  float2* gz = Gz + at;
+  float2* b = B + s.first;
+  float2* gy = Gy + s.first;
+  float2* gz = Gz + s.first;
   V u[E];
-#pragma unroll
-  for (int m = 0; m < E; ++m) u[m] = valid ? c_load<V>(b + m * (T * P)) : c_zero<V>();
-  // the Gz strip is read only by the third transform: start pulling it into L2 now
-  if (mem.w == 0 && valid) {
-#pragma unroll
-    for (int m = 0; m < E; ++m) prefetch_l2_line(gz + m * (T * P));
-  }
-  __syncwarp();
+  mem.collect(u, b, step, s.valid);
   park_store(park, u);
 #pragma unroll
   for (int m = 0; m < E; ++m) {
@@ -412,24 +519,30 @@ __device__ __forceinline__ void y_inv3_body(float2* __restrict__ B, float2* __re
     u[m] = mul_ik(u[m], (n == N / 2) ? 0.0f : kf * (float)signed_mode(n, N));
   }
   fft_regs<N, 1, true, C>(u, t, stw, mem);
-  if (valid) {
+  if (s.valid) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) c_store(gy + m * (T * P), u[m]);
+    for (int m = 0; m < E; ++m) c_store(gy + m * step, u[m]);
   }
   __syncwarp();
   park_load(park, u);
-  fft_regs<N, 1, true, C>(u, t, stw, mem);
-  if (valid) {
+  auto fetch_gz = [&] {
+    mem.sync();
+    mem.fetch(gz, step, s.valid);
+  };
+  fft_regs<N, 1, true, C>(u, t, stw, mem, fetch_gz);
+  if (s.valid) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) c_store(b + m * (T * P), u[m]);
-#pragma unroll
-    for (int m = 0; m < E; ++m) u[m] = c_load<V>(gz + m * (T * P));
+    for (int m = 0; m < E; ++m) c_store(b + m * step, u[m]);
   }
-  __syncwarp();
-  fft_regs<N, 1, true, C>(u, t, stw, mem);
-  if (valid) {
+  mem.collect(u, gz, step, s.valid);
+  auto after_reads = [&] {
+    mem.sync();
+    next();
+  };
+  fft_regs<N, 1, true, C>(u, t, stw, mem, after_reads);
+  if (s.valid) {
 #pragma unroll
-    for (int m = 0; m < E; ++m) c_store(gz + m * (T * P), u[m]);
+    for (int m = 0; m < E; ++m) c_store(gz + m * step, u[m]);
   }
   __syncwarp();
 }

@@ -11,6 +11,7 @@
 //   5. k_fft_x_c2r3     inverse x passes of (i k_x C, Gy, Gz') -> the three real force meshes
 // Steps 3-5 use linearity: i k_x and i k_y are constant along z, so the x and y components
 // share the inverse z transform of phi_k, and the x component shares the inverse y transform.
+#include "cols_launch.cuh"
 #include "pm_bodies.cuh"
 
 namespace cola {
@@ -53,33 +54,44 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * TY * TZ, deposit_min_block
   }
 }
 
+template <class Cfg>
+using ColsPark = TmemPark<Cfg::THREADS, Cfg::WORDS>;
+
 template <int N>
-using ColsPark = Park<cols_threads<N>(), FFTConf<N>::E, cpair>;
-template <int N>
-__global__ void __launch_bounds__(cols_threads<N>(), cols_min_blocks<N>())
+__global__ void __launch_bounds__(ColsCfg<N, kColsZ>::THREADS, ColsCfg<N, kColsZ>::MIN_BLOCKS)
     k_fft_z_green(float2* __restrict__ A, float2* __restrict__ Gz, float kf, int deconv, float norm,
                   const float2* __restrict__ tw) {
   extern __shared__ __align__(16) float2 sm[];
   __shared__ uint32_t slot;
-  const ColsPark<N> park(&slot);
-  constexpr int SL = cols_slabs<N>();
-  z_green_body<N, cols_width<N>(), SL, cpair>(A, Gz, kf, deconv, norm, tw, blockIdx.x, blockIdx.y * SL, sm, park);
+  using Cfg = ColsCfg<N, kColsZ>;
+  constexpr int P = half_pitch<N>();
+  float2* stab = sm + Cfg::TABLE;
+  float* sinc2 = reinterpret_cast<float*>(stab + stw_size<FFTConf<N>>());
+  stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
+  sinc2_fill<N>(sinc2, threadIdx.x, Cfg::THREADS);
+  const ColsPark<Cfg> park(&slot);  // (its block barrier publishes the tables as well)
+  const SmemTw<FFTConf<N>> stw{stab};
+  cols_walk<Cfg>(A, P, (int64_t)N * P, N, sm, [&](const auto& s, const auto& mem, auto& next) {
+    z_green_strip(A, Gz, kf, deconv, norm, stw, sinc2, s, mem, park, next);
+  });
   park.close();
-}
-template <int N>
-constexpr size_t z_smem() {
-  return sizeof(float2) * (z_table_offset<N, cols_width<N>(), cols_slabs<N>()>() + stw_size<FFTConf<N>>());
 }
 
 template <int N>
-__global__ void __launch_bounds__(cols_threads<N>(), cols_min_blocks<N>())
+__global__ void __launch_bounds__(ColsCfg<N, kColsY>::THREADS, ColsCfg<N, kColsY>::MIN_BLOCKS)
     k_fft_y_inv3(float2* __restrict__ B, float2* __restrict__ Gy, float2* __restrict__ Gz, float kf,
                  const float2* __restrict__ tw) {
   extern __shared__ __align__(16) float2 sm[];
   __shared__ uint32_t slot;
-  const ColsPark<N> park(&slot);
-  constexpr int SL = cols_slabs<N>();
-  y_inv3_body<N, cols_width<N>(), SL, cpair>(B, Gy, Gz, kf, tw, blockIdx.x, blockIdx.y * SL, sm, park);
+  using Cfg = ColsCfg<N, kColsY>;
+  constexpr int P = half_pitch<N>();
+  float2* stab = sm + Cfg::TABLE;
+  stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
+  const ColsPark<Cfg> park(&slot);
+  const SmemTw<FFTConf<N>> stw{stab};
+  cols_walk<Cfg>(B, (int64_t)N * P, P, N, sm, [&](const auto& s, const auto& mem, auto& next) {
+    y_inv3_strip(B, Gy, Gz, kf, stw, s, mem, park, next);
+  });
   park.close();
 }
 
@@ -195,7 +207,7 @@ template <int N>
 static int force_passes_t(const Geometry& g, const Tiles& tl, const uint4* rec, const int* offsets,
                           float2* A, float2* Gy, float2* Gz, float* F, int P, double box, int deconv,
                           const float2* tw, int* err, cudaStream_t st) {
-  constexpr int M = N / 2, W = cols_width<N>(), nh = N / 2 + 1;
+  constexpr int M = N / 2, nh = N / 2 + 1;
   const float kf = (float)(2.0 * 3.14159265358979323846 / box);
   const float norm = (float)(1.0 / ((double)N * N * N));
   if (P != half_pitch<N>()) return fail(COLA_EINVAL, "force passes: unexpected half-spectrum pitch");
@@ -203,22 +215,23 @@ static int force_passes_t(const Geometry& g, const Tiles& tl, const uint4* rec, 
   if ((rc = deposit_fftx_t<N>(g, tl, rec, offsets, A, P, tw, err, st))) return rc;
   // 2. forward y pass
   if ((rc = launch_fft_cols(N, false, A, N, (int64_t)N * P, P, nh, tw, st))) return rc;
-  constexpr int SL = cols_slabs<N>();
-  const dim3 grid((nh + W - 1) / W, N / SL);
+  unsigned grid = 0;
   // 3. z pass with the Green's function
   {
-    constexpr size_t smem = z_smem<N>();
-    if ((rc = set_smem(k_fft_z_green<N>, smem))) return rc;
+    using Cfg = ColsCfg<N, kColsZ>;
+    constexpr size_t smem = cols_smem<Cfg>(N);
+    if ((rc = cols_grid<Cfg, k_fft_z_green<N>>(smem, Cfg::STRIPS * N, &grid))) return rc;
     LaunchScope ls_(flabel<N>(1), st);
-    k_fft_z_green<N><<<grid, cols_threads<N>(), smem, st>>>(A, Gz, kf, deconv, norm, tw);
+    k_fft_z_green<N><<<grid, Cfg::THREADS, smem, st>>>(A, Gz, kf, deconv, norm, tw);
     COLA_LAUNCH_CHECK();
   }
   // 4. inverse y passes
   {
-    constexpr size_t smem = sizeof(float2) * (SL * N * W + stw_size<FFTConf<N>>());
-    if ((rc = set_smem(k_fft_y_inv3<N>, smem))) return rc;
+    using Cfg = ColsCfg<N, kColsY>;
+    constexpr size_t smem = cols_smem<Cfg>(0);
+    if ((rc = cols_grid<Cfg, k_fft_y_inv3<N>>(smem, Cfg::STRIPS * N, &grid))) return rc;
     LaunchScope ls_(flabel<N>(2), st);
-    k_fft_y_inv3<N><<<grid, cols_threads<N>(), smem, st>>>(A, Gy, Gz, kf, tw);
+    k_fft_y_inv3<N><<<grid, Cfg::THREADS, smem, st>>>(A, Gy, Gz, kf, tw);
     COLA_LAUNCH_CHECK();
   }
   // 5. inverse x passes (persistent, bulk-copy pipelined)

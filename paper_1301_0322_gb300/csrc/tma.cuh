@@ -60,10 +60,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return true;
 }
 
-// Prefetch the L2 line holding `p` (a hint; no completion to wait for).
-__device__ __forceinline__ void prefetch_l2_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-// drop the 128-byte L2 line at p (128-byte aligned) without writing it back: for scratch that
-// is dead until its next writer overwrites it whole
-__device__ __forceinline__ void discard_l2_line(void* p) { asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory"); }
+// 16 bytes from global memory straight into shared memory (past the L1 cache: a load that goes
+// through it holds a 128-byte line until it returns, and kernels that take most of the SM's
+// memory as shared memory leave few lines), zeros if !valid; completed by copy_wait_all
+__device__ __forceinline__ void copy_async16(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(valid ? 16 : 0)
+               : "memory");
+}
+// this thread's asynchronous copies have arrived (visible to this thread)
+__device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 
 }  // namespace cola
