@@ -158,8 +158,8 @@ void twiddle_table(int n, std::vector<float2>& out);
 int launch_fft_x_r2c(int n, const float* in, float2* out, int64_t nrows, int P, const float2* tw, cudaStream_t st);
 int launch_fft_x_c2r(int n, const float2* in, float* out, int64_t nrows, int P, const float2* tw, float scale,
                      cudaStream_t st);
-int launch_fft_cols(int n, bool inverse, float2* data, int64_t nslabs, int64_t slab_stride, int64_t row_stride,
-                    int ncols, const float2* tw, cudaStream_t st);
+// in place over a half spectrum [n][n][P], along y or along z
+int launch_fft_cols(int n, bool inverse, bool along_z, float2* data, int P, const float2* tw, cudaStream_t st);
 // 3-D helpers built on the passes: r2c (x then y then z) and c2r (z, y, x), layout [n][n][P]
 int fft3d_r2c(int n, int P, const float* in, float2* out, const float2* tw, cudaStream_t st);
 int fft3d_c2r(int n, int P, float2* in_destroyed, float* out, const float2* tw, float scale, cudaStream_t st);

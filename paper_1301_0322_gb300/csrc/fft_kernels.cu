@@ -16,18 +16,19 @@ __host__ __device__ constexpr int x_rows() {
   return FFTConf<N / 2>::T >= 256 ? 1 : 256 / FFTConf<N / 2>::T;
 }
 
-// In-place FFT of the N/2 + 1 columns of nslabs slabs: element (n, col) at data[slab*slab_stride + n*row_stride + col].
-template <int N, bool INV>
+// In-place FFT of the N/2 + 1 columns of the N slabs of a half spectrum, along y (slab = z) or
+// along z (slab = y).
+template <int N, bool INV, bool ALONG_Z>
 __global__ void __launch_bounds__(ColsCfg<N, kColsPlain>::THREADS, ColsCfg<N, kColsPlain>::MIN_BLOCKS)
-    k_fft_cols(float2* __restrict__ data, int64_t slab_stride, int64_t row_stride, int nslabs,
-               const float2* __restrict__ tw) {
+    k_fft_cols(float2* __restrict__ data, const float2* __restrict__ tw) {
   extern __shared__ __align__(16) float2 smem[];
   using Cfg = ColsCfg<N, kColsPlain>;
   float2* stab = smem + Cfg::TABLE;
   stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
   __syncthreads();
   const SmemTw<FFTConf<N>> stw{stab};
-  cols_walk<Cfg>(data, slab_stride, row_stride, nslabs, smem,
+  constexpr int64_t P = half_pitch<N>();
+  cols_walk<Cfg>(data, ALONG_Z ? P : N * P, ALONG_Z ? N * P : P, N, smem,
                  [&](const auto& s, const auto& mem, auto& next) { cols_strip<INV>(data, s, stw, mem, next); });
 }
 
@@ -136,26 +137,22 @@ static int x_c2r(const float2* in, float* out, int64_t nrows, int P, const float
   return COLA_OK;
 }
 
-template <int N>
-static int cols(bool inverse, float2* data, int64_t nslabs, int64_t slab_stride, int64_t row_stride, int ncols,
-                const float2* tw, cudaStream_t st) {
-  if (nslabs > 65535 || ncols != N / 2 + 1) return fail(COLA_EINVAL, "fft column pass: unexpected slabs or columns");
+template <int N, bool INV, bool ALONG_Z>
+static int cols_t(float2* data, const float2* tw, cudaStream_t st) {
   using Cfg = ColsCfg<N, kColsPlain>;
-  const int64_t strips = Cfg::STRIPS * nslabs;
   constexpr size_t smem = cols_smem<Cfg>(0);
   unsigned grid = 0;
-  int rc;
-  if (inverse) {
-    if ((rc = cols_grid<Cfg, k_fft_cols<N, true>>(smem, strips, &grid))) return rc;
-    LaunchScope ls_(label<N>("inv"), st);
-    k_fft_cols<N, true><<<grid, Cfg::THREADS, smem, st>>>(data, slab_stride, row_stride, (int)nslabs, tw);
-  } else {
-    if ((rc = cols_grid<Cfg, k_fft_cols<N, false>>(smem, strips, &grid))) return rc;
-    LaunchScope ls_(label<N>("fwd"), st);
-    k_fft_cols<N, false><<<grid, Cfg::THREADS, smem, st>>>(data, slab_stride, row_stride, (int)nslabs, tw);
-  }
+  if (const int rc = cols_grid<Cfg, k_fft_cols<N, INV, ALONG_Z>>(smem, Cfg::STRIPS * N, &grid)) return rc;
+  LaunchScope ls_(label<N>(INV ? "inv" : "fwd"), st);
+  k_fft_cols<N, INV, ALONG_Z><<<grid, Cfg::THREADS, smem, st>>>(data, tw);
   COLA_LAUNCH_CHECK();
   return COLA_OK;
+}
+template <int N>
+static int cols(bool inverse, bool along_z, float2* data, int P, const float2* tw, cudaStream_t st) {
+  if (P != half_pitch<N>()) return fail(COLA_EINVAL, "fft column pass: unexpected row pitch");
+  if (inverse) return along_z ? cols_t<N, true, true>(data, tw, st) : cols_t<N, true, false>(data, tw, st);
+  return along_z ? cols_t<N, false, true>(data, tw, st) : cols_t<N, false, false>(data, tw, st);
 }
 
 #define COLA_FOR_SIZES(X) \
@@ -197,12 +194,11 @@ int launch_fft_x_c2r(int n, const float2* in, float* out, int64_t nrows, int P, 
   }
 }
 
-int launch_fft_cols(int n, bool inverse, float2* data, int64_t nslabs, int64_t slab_stride, int64_t row_stride,
-                    int ncols, const float2* tw, cudaStream_t st) {
+int launch_fft_cols(int n, bool inverse, bool along_z, float2* data, int P, const float2* tw, cudaStream_t st) {
   switch (n) {
 #define X(N) \
   case N:    \
-    return cols<N>(inverse, data, nslabs, slab_stride, row_stride, ncols, tw, st);
+    return cols<N>(inverse, along_z, data, P, tw, st);
     COLA_FOR_SIZES(X)
 #undef X
     default:
@@ -214,16 +210,16 @@ int fft3d_r2c(int n, int P, const float* in, float2* out, const float2* tw, cuda
   const int64_t nn = n;
   int rc = launch_fft_x_r2c(n, in, out, nn * nn, P, tw, st);
   if (rc) return rc;
-  rc = launch_fft_cols(n, false, out, nn, nn * P, P, n / 2 + 1, tw, st);  // y: slab = z
+  rc = launch_fft_cols(n, false, false, out, P, tw, st);
   if (rc) return rc;
-  return launch_fft_cols(n, false, out, nn, P, nn * P, n / 2 + 1, tw, st);  // z: slab = y
+  return launch_fft_cols(n, false, true, out, P, tw, st);
 }
 
 int fft3d_c2r(int n, int P, float2* in, float* out, const float2* tw, float scale, cudaStream_t st) {
   const int64_t nn = n;
-  int rc = launch_fft_cols(n, true, in, nn, P, nn * P, n / 2 + 1, tw, st);  // z
+  int rc = launch_fft_cols(n, true, true, in, P, tw, st);
   if (rc) return rc;
-  rc = launch_fft_cols(n, true, in, nn, nn * P, P, n / 2 + 1, tw, st);  // y
+  rc = launch_fft_cols(n, true, false, in, P, tw, st);
   if (rc) return rc;
   return launch_fft_x_c2r(n, in, out, nn * nn, P, tw, scale, st);
 }

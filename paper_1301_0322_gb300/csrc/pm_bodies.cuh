@@ -91,7 +91,8 @@ template <int N, int KIND>
 struct ColsCfg {
   using C = FFTConf<N>;
   static constexpr int N_ = N;
-  // two columns per thread from 256 up; below, one, on twice the threads
+  // two columns per thread from 256 up; below, one, on twice the threads (256: z 57 us, 70 with
+  // one; 192: z 33, 35-39 with two)
   using V = std::conditional_t<(N >= 256), cpair, float2>;
   // 16 columns are 128-byte row segments; 8 where buffers of 16 do not fit
   static constexpr int W = (N >= 1536 || (N == 768 && KIND == kColsY)) ? 8 : 16;
@@ -108,7 +109,8 @@ struct ColsCfg {
                                 : N == 768  ? (KIND == kColsZ ? 512 : 256)
                                 : N == 512  ? 1024
                                 : N == 384  ? (KIND == kColsPlain ? 256 : 384)
-                                            : 512;
+                                : N == 256  ? 512
+                                            : 256;
   // persistent blocks, one wave of them, from 384 up
   static constexpr bool RESIDENT = N >= 384;
   static constexpr int K = lanes_of<V>(), GROUP = C::T * W / K, THREADS = GROUP * G;

@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * TY * TZ, deposit_min_block
 }
 
 template <class Cfg>
-using ColsPark = TmemPark<Cfg::THREADS, Cfg::WORDS>;
+using ColsPark = std::conditional_t<Cfg::K == 1, RegPark<Cfg::WORDS>, TmemPark<Cfg::THREADS, Cfg::WORDS>>;
 
 template <int N>
 __global__ void __launch_bounds__(ColsCfg<N, kColsZ>::THREADS, ColsCfg<N, kColsZ>::MIN_BLOCKS)
@@ -207,14 +207,14 @@ template <int N>
 static int force_passes_t(const Geometry& g, const Tiles& tl, const uint4* rec, const int* offsets,
                           float2* A, float2* Gy, float2* Gz, float* F, int P, double box, int deconv,
                           const float2* tw, int* err, cudaStream_t st) {
-  constexpr int M = N / 2, nh = N / 2 + 1;
+  constexpr int M = N / 2;
   const float kf = (float)(2.0 * 3.14159265358979323846 / box);
   const float norm = (float)(1.0 / ((double)N * N * N));
   if (P != half_pitch<N>()) return fail(COLA_EINVAL, "force passes: unexpected half-spectrum pitch");
   int rc;
   if ((rc = deposit_fftx_t<N>(g, tl, rec, offsets, A, P, tw, err, st))) return rc;
   // 2. forward y pass
-  if ((rc = launch_fft_cols(N, false, A, N, (int64_t)N * P, P, nh, tw, st))) return rc;
+  if ((rc = launch_fft_cols(N, false, false, A, P, tw, st))) return rc;
   unsigned grid = 0;
   // 3. z pass with the Green's function
   {
@@ -270,8 +270,8 @@ int launch_density_spectrum(const Geometry& g, const Tiles& tl, const uint4* rec
   case N: {                                                                                           \
     int rc;                                                                                           \
     if ((rc = deposit_fftx_t<N>(g, tl, rec, offsets, A, P, tw, err, st))) return rc;                  \
-    if ((rc = launch_fft_cols(N, false, A, N, (int64_t)N * P, P, N / 2 + 1, tw, st))) return rc;      \
-    return launch_fft_cols(N, false, A, N, P, (int64_t)N * P, N / 2 + 1, tw, st); /* z: slab = y */ \
+    if ((rc = launch_fft_cols(N, false, false, A, P, tw, st))) return rc;                                       \
+    return launch_fft_cols(N, false, true, A, P, tw, st);                                              \
   }
     X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768) X(1024) X(1536) X(2048)
 #undef X

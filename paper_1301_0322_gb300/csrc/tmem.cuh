@@ -99,6 +99,24 @@ struct TmemPark {
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "n"(COLS) : "memory");
   }
 };
+// The same in the thread's own registers, for transforms short enough to leave room for a copy.
+template <int MAX>
+struct RegPark {
+  mutable uint32_t kept[MAX];
+  __device__ __forceinline__ explicit RegPark(uint32_t*) { __syncthreads(); }
+  template <int N>
+  __device__ __forceinline__ void store(const uint32_t (&r)[N]) const {
+    static_assert(N <= MAX, "this thread's words");
+#pragma unroll
+    for (int i = 0; i < N; ++i) kept[i] = r[i];
+  }
+  template <int N>
+  __device__ __forceinline__ void load(uint32_t (&r)[N]) const {
+#pragma unroll
+    for (int i = 0; i < N; ++i) r[i] = kept[i];
+  }
+  __device__ __forceinline__ void close() const {}
+};
 // for a kernel that parks nothing
 struct NoPark {
   __device__ __forceinline__ explicit NoPark(uint32_t*) {}
