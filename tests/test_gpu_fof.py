@@ -104,3 +104,22 @@ def test_fof_stays_inside_its_workspace(cola, n_p, ng):
     binding.cola_status(h)
     assert bool((buf[nbytes:] == 0x5A).all())
     binding.cola_plan_destroy(h)
+
+
+@pytest.mark.parametrize("n_p,ng,b,kind", [(32, 32, (1, 5), "clumps"), (32, 64, (1, 1), "random"), (32, 192, (1, 5), "clumps"),
+                                           (48, 96, (1, 6), "clumps"), (32, 96, (3, 5), "random"), (32, 64, (1, 5), "one cell")])
+def test_fof_linking_cells(cola, n_p, ng, b, kind):
+    # cells of one and of several mesh cells, groups across the faces of the box, and every particle
+    # in a few cells (more candidates than a particle has lanes)
+    box = 40.0
+    if kind == "clumps":
+        s32 = inputs.clustered_displacements(n_p, box, 7)
+    elif kind == "random":
+        s32 = inputs.gaussian_displacements(n_p, box, 8)
+    else:
+        p = np.arange(n_p**3)
+        q = np.stack([p % n_p, (p // n_p) % n_p, p // (n_p * n_p)]) * (box / n_p)
+        away = np.random.default_rng(9).normal(0, 0.15 * box / n_p, size=q.shape)
+        pull = p % 29 == 0  # a clump around the corner of the box, the others stay near the lattice
+        s32 = np.where(pull, np.where(q > box / 2, box - q, -q) + away, 0.1 * away).astype(np.float32)
+    check(cola, cola.Plan(np_side=n_p, ng=ng, box=box), s32, n_p, ng, box, b=b, nmin=5)
