@@ -292,7 +292,20 @@ __device__ __forceinline__ void cols_walk(const float2* src, int64_t slab_stride
 // rows' transform buffers); ints: 28 ints of shared memory
 // rec: the bin-ordered particle records (fixed-point CIC coordinates; offsets index them directly)
 // (stw: the row transform's stage twiddles, the base table tw or an SmemTw table)
-template <int N, int TY, int TZ, class CM = FFTConf<N / 2>, class STW>
+// The block has D >= T(N/2) TY TZ threads: all of them deposit, the first T(N/2) TY TZ transform.
+// Row buffers of a tile, with a barrier of their own for the threads that transform:
+template <int R0, int NT, int D>
+struct RowBuffer {
+  float2* buf;
+  __device__ __forceinline__ float2& operator()(int n) const { return buf[xpad<R0>(n)]; }
+  __device__ __forceinline__ void sync() const {
+    if constexpr (NT == D) __syncthreads();
+    else if constexpr (NT < 32) __syncwarp((1u << NT) - 1u);
+    else if constexpr (NT == 32) __syncwarp();
+    else asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+  }
+};
+template <int N, int TY, int TZ, class CM = FFTConf<N / 2>, int D = CM::T * TY * TZ, class STW>
 __device__ __forceinline__ void deposit_fftx_body(const Geometry& g, const Tiles& tl, const uint4* __restrict__ rec,
                                                   const int* __restrict__ offsets, float2* __restrict__ out, int P,
                                                   const float2* __restrict__ tw, const STW& stw, float dscale,
@@ -305,10 +318,10 @@ __device__ __forceinline__ void deposit_fftx_body(const Geometry& g, const Tiles
   int tyi, tzi;
   tile_of_bin(tl, tile, tyi, tzi);
   const int y0 = tyi * TY, z0 = tzi * TZ;
-  for (int i = threadIdx.x; i < ROWS * N; i += NT) acc[i] = 0ull;
+  for (int i = threadIdx.x; i < ROWS * N; i += D) acc[i] = 0ull;
   // the tile's own 4 bins and the boundary bins of its 3 lower neighbours, loaded in parallel
-  // (a loop: at N = 32 and 48 a block has only 8 threads)
-  for (int k = threadIdx.x; k < 9; k += NT) {
+  // (a loop: a block may have fewer than 9 threads)
+  for (int k = threadIdx.x; k < 9; k += D) {
     const int tym = tyi == 0 ? tl.nty - 1 : tyi - 1;
     const int tzm = tzi == 0 ? tl.ntz - 1 : tzi - 1;
     const int ty_ = (k == 4 || k == 5 || k == 8) ? tym : tyi;
@@ -330,17 +343,15 @@ __device__ __forceinline__ void deposit_fftx_body(const Geometry& g, const Tiles
   }
   __syncthreads();
   const int total = rpre[9];
-  const unsigned long long one = 1ull << g.fbits;
   unsigned* lo = reinterpret_cast<unsigned*>(acc);
   unsigned* hi = lo + ROWS * N;
   constexpr int U = 4;  // particles in flight per thread
-  const uint32_t fmask = (uint32_t)one - 1u;
-  for (int base = threadIdx.x; base < total; base += NT * U) {
+  for (int base = threadIdx.x; base < total; base += D * U) {
     uint32_t f[U][3];
     bool ok[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = base + u * NT;
+      const int i = base + u * D;
       ok[u] = i < total;
       if (ok[u]) {
         int r = 0;
@@ -353,38 +364,19 @@ __device__ __forceinline__ void deposit_fftx_body(const Geometry& g, const Tiles
       }
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (!ok[u]) continue;
-      const int cx = (int)(f[u][0] >> g.fbits), tx = (int)(f[u][0] & fmask);
-      const int cy = (int)(f[u][1] >> g.fbits), ty = (int)(f[u][1] & fmask);
-      const int cz = (int)(f[u][2] >> g.fbits), tz = (int)(f[u][2] & fmask);
-      const int cx1 = wrap_inc(cx, N);
-      const unsigned long long wx0 = one - tx, wx1 = tx;
-#pragma unroll
-      for (int dz = 0; dz < 2; ++dz) {
-        const int lz = (dz ? wrap_inc(cz, N) : cz) - z0;
-        if (lz < 0 || lz >= TZ) continue;
-        const unsigned long long wz = dz ? (unsigned long long)tz : one - tz;
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy) {
-          const int ly = (dy ? wrap_inc(cy, N) : cy) - y0;
-          if (ly < 0 || ly >= TY) continue;
-          const unsigned long long wzy = wz * (dy ? (unsigned long long)ty : one - ty);
-          const int row = (lz * TY + ly) * N;
-          acc_add64(lo, hi, row + cx, wzy * wx0);
-          acc_add64(lo, hi, row + cx1, wzy * wx1);
-        }
-      }
-    }
+    for (int u = 0; u < U; ++u)
+      if (ok[u]) acc_cloud<TY, TZ, (N <= 384)>(lo, hi, f[u], g.fbits, N, y0, z0);
   }
   __syncthreads();
   // real-to-complex FFT of each tile row; z[n] = (delta[2n], delta[2n+1]).  The transform
   // buffers overlay the accumulators: fft_1d reads all its inputs before a block barrier
   // that precedes its first shared-memory write.
+  if (NT < D && (int)threadIdx.x >= NT) return;
   const int t = threadIdx.x % T, w = threadIdx.x / T;
   const uint2* lrow = reinterpret_cast<const uint2*>(lo + w * N);
   const uint2* hrow = reinterpret_cast<const uint2*>(hi + w * N);
   float2* buf = reinterpret_cast<float2*>(acc) + w * LD;
+  RowBuffer<R0, NT, D> mem{buf};
   bool overflow = false;
   auto load = [&](int n) -> float2 {
     const uint2 l = lrow[n], h = hrow[n];
@@ -393,11 +385,10 @@ __device__ __forceinline__ void deposit_fftx_body(const Geometry& g, const Tiles
     const unsigned long long b = ((unsigned long long)h.y << 32) | l.y;
     return make_float2(fmaf(u64_to_f32_rn(a), dscale, -1.0f), fmaf(u64_to_f32_rn(b), dscale, -1.0f));
   };
-  auto mem = [&](int n) -> float2& { return buf[xpad<R0>(n)]; };
   auto store = [&](int n, float2 x) { buf[xpad<R0>(n)] = x; };
   fft_1d<M, 2, false, CM>(t, stw, load, mem, store);
   if (overflow) atomicOr(err, kErrOverflow);
-  __syncthreads();
+  mem.sync();
   const int lz = w / TY, ly = w - lz * TY;
   float2* dst = out + ((int64_t)(z0 + lz) * N + (y0 + ly)) * P;
   // X[k] and X[M - k] from one pair Z[k], Z[M - k]: with e = (Z[k] + conj Z[M - k]) / 2,

@@ -17,11 +17,22 @@
 namespace cola {
 
 // ---- single-box kernels ------------------------------------------------------------------------
-// resident blocks per SM the fused deposit is compiled for: 512 threads per SM, and three blocks
-// of 2 x 2 tiles at N = 2048 (64 KB of cell sums each; 80 registers, no spills)
+// Threads of the fused deposit: those of the row transforms (8 to 128 for 8 rows), and up to 256
+// cells per side more to deposit with: there a tile with a clump in it keeps the few threads of its
+// transforms busy long after the other tiles are done.  us per launch with the transforms' threads
+// alone -> these: 32^3 mesh and particles 117 -> 11, 64: 16 -> 8, 192 with clumps 78 -> 39, 256 with
+// clumps 272 -> 219 (without 76 either way); at 384 128 threads lose (250 -> 263).
+template <int N, int TY, int TZ>
+__host__ __device__ constexpr int deposit_threads() {
+  constexpr int rows = FFTConf<N / 2>::T * TY * TZ, least = N <= 96 ? 256 : (N <= 256 ? 128 : 0);
+  return rows < least ? least : rows;
+}
+// resident blocks per SM it is compiled for, by threads per SM; three blocks of 2 x 2 tiles at
+// N = 2048 (64 KB of cell sums each; 80 registers, no spills)
 template <int N, int TY, int TZ>
 __host__ __device__ constexpr int deposit_min_blocks() {
-  return N == 2048 && TY * TZ == 4 ? 3 : ((512 / (FFTConf<N / 2>::T * TY * TZ)) > 0 ? 512 / (FFTConf<N / 2>::T * TY * TZ) : 1);
+  constexpr int per_sm = (N <= 96 ? 1024 : (N <= 256 ? 768 : 512)) / deposit_threads<N, TY, TZ>();
+  return N == 2048 && TY * TZ == 4 ? 3 : (per_sm > 0 ? per_sm : 1);
 }
 
 // cell sums (8 bytes per cell) of a TY x TZ tile, which later hold the rows' transform buffers
@@ -38,7 +49,7 @@ __host__ __device__ constexpr int deposit_table_size() {
 }
 
 template <int N, int TY, int TZ>
-__global__ void __launch_bounds__(FFTConf<N / 2>::T * TY * TZ, deposit_min_blocks<N, TY, TZ>())
+__global__ void __launch_bounds__(deposit_threads<N, TY, TZ>(), deposit_min_blocks<N, TY, TZ>())
     k_deposit_fftx(Geometry g, Tiles tl, const uint4* __restrict__ rec, const int* __restrict__ offsets,
                    float2* __restrict__ out, int P, const float2* __restrict__ tw, float dscale,
                    int* __restrict__ err) {
@@ -47,10 +58,11 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * TY * TZ, deposit_min_block
   if constexpr (deposit_table_size<N>() > 0) {
     float2* stab = reinterpret_cast<float2*>(acc + deposit_acc_cells<N, TY, TZ>());
     stw_fill<FFTConf<N / 2>, 2, true>(stab, tw, threadIdx.x, blockDim.x);
-    deposit_fftx_body<N, TY, TZ>(g, tl, rec, offsets, out, P, tw, SmemTw<FFTConf<N / 2>, true>{stab}, dscale, err,
-                                 blockIdx.x, acc, ints);
+    deposit_fftx_body<N, TY, TZ, FFTConf<N / 2>, deposit_threads<N, TY, TZ>()>(
+        g, tl, rec, offsets, out, P, tw, SmemTw<FFTConf<N / 2>, true>{stab}, dscale, err, blockIdx.x, acc, ints);
   } else {
-    deposit_fftx_body<N, TY, TZ>(g, tl, rec, offsets, out, P, tw, tw, dscale, err, blockIdx.x, acc, ints);
+    deposit_fftx_body<N, TY, TZ, FFTConf<N / 2>, deposit_threads<N, TY, TZ>()>(g, tl, rec, offsets, out, P, tw, tw,
+                                                                               dscale, err, blockIdx.x, acc, ints);
   }
 }
 
@@ -180,7 +192,6 @@ static const char* flabel(int kind) {
 template <int N>
 static int deposit_fftx_t(const Geometry& g, const Tiles& tl, const uint4* rec, const int* offsets, float2* A, int P,
                           const float2* tw, int* err, cudaStream_t st) {
-  constexpr int M = N / 2;
   int rc;
   const double n3 = (double)N * N * N;
   const float dscale = (float)(n3 / ((double)g.np3 * std::ldexp(1.0, 3 * g.fbits)));
@@ -188,13 +199,13 @@ static int deposit_fftx_t(const Geometry& g, const Tiles& tl, const uint4* rec, 
     const size_t smem = sizeof(unsigned long long) * (deposit_acc_cells<N, 4, 2>() + deposit_table_size<N>());
     if ((rc = set_smem(k_deposit_fftx<N, 4, 2>, smem))) return rc;
     LaunchScope ls_(flabel<N>(0), st);
-    k_deposit_fftx<N, 4, 2><<<tl.nty * tl.ntz, FFTConf<M>::T * 8, smem, st>>>(g, tl, rec, offsets, A, P, tw,
+    k_deposit_fftx<N, 4, 2><<<tl.nty * tl.ntz, deposit_threads<N, 4, 2>(), smem, st>>>(g, tl, rec, offsets, A, P, tw,
                                                                                 dscale, err);
   } else if (tl.ty == 2 && tl.tz == 2) {
     const size_t smem = sizeof(unsigned long long) * (deposit_acc_cells<N, 2, 2>() + deposit_table_size<N>());
     if ((rc = set_smem(k_deposit_fftx<N, 2, 2>, smem))) return rc;
     LaunchScope ls_(flabel<N>(0), st);
-    k_deposit_fftx<N, 2, 2><<<tl.nty * tl.ntz, FFTConf<M>::T * 4, smem, st>>>(g, tl, rec, offsets, A, P, tw,
+    k_deposit_fftx<N, 2, 2><<<tl.nty * tl.ntz, deposit_threads<N, 2, 2>(), smem, st>>>(g, tl, rec, offsets, A, P, tw,
                                                                                 dscale, err);
   } else {
     return fail(COLA_EUNSUPPORTED, "fused deposit: unsupported tile shape");

@@ -125,7 +125,6 @@ __global__ void __launch_bounds__(256) k_deposit(Geometry g, Tiles tl, const uin
   }
   __syncthreads();
   const int total = rpre[9];
-  const unsigned long long one = 1ull << g.fbits;
   unsigned* lo = reinterpret_cast<unsigned*>(acc);
   unsigned* hi = lo + ncell;
   for (int i = threadIdx.x; i < total; i += blockDim.x) {
@@ -133,31 +132,9 @@ __global__ void __launch_bounds__(256) k_deposit(Geometry g, Tiles tl, const uin
 #pragma unroll
     for (int k = 1; k < 9; ++k) r += (i >= rpre[k]) ? 1 : 0;
     const int64_t pos = rbeg[r] + (i - rpre[r]);
-    const uint32_t fmask = (uint32_t)one - 1u;
     const uint4 q = __ldg(rec + pos);
-    const uint32_t fx = q.x, fy = q.y, fz = q.z;
-    const int cx = (int)(fx >> g.fbits), tx = (int)(fx & fmask);
-    const int cy = (int)(fy >> g.fbits), ty = (int)(fy & fmask);
-    const int cz = (int)(fz >> g.fbits), tz = (int)(fz & fmask);
-    const int cx1 = wrap_inc(cx, ng);
-    const unsigned long long wx0 = one - tx, wx1 = tx;
-#pragma unroll
-    for (int dz = 0; dz < 2; ++dz) {
-      const int z = dz ? wrap_inc(cz, ng) : cz;
-      const int lz = z - z0;
-      if (lz < 0 || lz >= TZ) continue;
-      const unsigned long long wz = dz ? (unsigned long long)tz : one - tz;
-#pragma unroll
-      for (int dy = 0; dy < 2; ++dy) {
-        const int y = dy ? wrap_inc(cy, ng) : cy;
-        const int ly = y - y0;
-        if (ly < 0 || ly >= TY) continue;
-        const unsigned long long wzy = wz * (dy ? (unsigned long long)ty : one - ty);
-        const int row = (lz * TY + ly) * ng;
-        acc_add64(lo, hi, row + cx, wzy * wx0);
-        acc_add64(lo, hi, row + cx1, wzy * wx1);
-      }
-    }
+    const uint32_t f[3] = {q.x, q.y, q.z};
+    acc_cloud<TY, TZ, false>(lo, hi, f, g.fbits, ng, y0, z0);
   }
   __syncthreads();
   bool overflow = false;
