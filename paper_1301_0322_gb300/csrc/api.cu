@@ -296,27 +296,25 @@ int cola_ic_2lpt(cola_plan* plan, const float* noise, float* s, float* v, float*
     return rc;
   // s1 = i k delta / k^2
   for (int j = 0; j < 3; ++j) {
-    if ((rc = launch_kmul(n, P, box, 0, j, 0, norm, w.icC0, w.icC1, st))) return rc;
-    if ((rc = fft3d_c2r(n, P, w.icC1, s1 + j * n3, w.tw_p, 1.0f, st))) return rc;
+    if ((rc = fft3d_c2r_factor(n, P, box, 0, j, 0, norm, w.icC0, w.icC1, s1 + j * n3, false, w.tw_p, w.err, st)))
+      return rc;
   }
   // mu2 = psi_xx psi_yy + psi_xx psi_zz + psi_yy psi_zz - psi_xy^2 - psi_xz^2 - psi_yz^2
   for (int j = 0; j < 3; ++j) {
-    if ((rc = launch_kmul(n, P, box, 1, j, j, norm, w.icC0, w.icC1, st))) return rc;
-    if ((rc = fft3d_c2r(n, P, w.icC1, w.icR[j], w.tw_p, 1.0f, st))) return rc;
+    if ((rc = fft3d_c2r_factor(n, P, box, 1, j, j, norm, w.icC0, w.icC1, w.icR[j], false, w.tw_p, w.err, st))) return rc;
   }
   if ((rc = launch_source_2lpt(n3, w.icR[0], w.icR[1], w.icR[2], w.icR[0], st))) return rc;
   const int pairs[3][2] = {{0, 1}, {0, 2}, {1, 2}};
   for (auto& ij : pairs) {
-    if ((rc = launch_kmul(n, P, box, 1, ij[0], ij[1], norm, w.icC0, w.icC1, st))) return rc;
-    if ((rc = fft3d_c2r(n, P, w.icC1, w.icR[1], w.tw_p, 1.0f, st))) return rc;
-    if ((rc = launch_source_sub_sq(n3, w.icR[1], w.icR[0], st))) return rc;
+    if ((rc = fft3d_c2r_factor(n, P, box, 1, ij[0], ij[1], norm, w.icC0, w.icC1, w.icR[0], true, w.tw_p, w.err, st)))
+      return rc;
   }
   // s2 = D2u(1) * (-i k mu2_k / k^2)
   if ((rc = fft3d_r2c(n, P, w.icR[0], w.icC1, w.tw_p, st))) return rc;
   const float s2scale = (float)(-plan->d2u1 / (double)n3);
   for (int j = 0; j < 3; ++j) {
-    if ((rc = launch_kmul(n, P, box, 0, j, 0, s2scale, w.icC1, w.icC0, st))) return rc;
-    if ((rc = fft3d_c2r(n, P, w.icC0, s2 + j * n3, w.tw_p, 1.0f, st))) return rc;
+    if ((rc = fft3d_c2r_factor(n, P, box, 0, j, 0, s2scale, w.icC1, w.icC0, s2 + j * n3, false, w.tw_p, w.err, st)))
+      return rc;
   }
   // v = T[s] after L- (eq. Lops): 0 in the LPT frame; the standard leapfrog starts from the
   // full 2LPT velocity T[D1] s1 + T[D2] s2
@@ -477,7 +475,7 @@ int cola_step_adjoint(cola_plan* plan, int32_t step, const float* s_ckpt, float*
   if ((rc = launch_kspace_adjoint(ng, plan->Pg, plan->cfg.box, plan->cfg.deconv, half[0], half[1], half[2], st)))
     return rc;
   float* phi = w.lam_real;
-  if ((rc = fft3d_c2r(ng, plan->Pg, half[0], phi, w.tw_g, 1.0f, st))) return rc;
+  if ((rc = fft3d_c2r(ng, plan->Pg, half[0], phi, w.tw_g, 1.0f, w.err, st))) return rc;
   const double* row = &plan->coef64[(size_t)step * COLA_NCOEF];
   const double to_cells = (double)ng / plan->cfg.box;
   const double inv_rho_bar = (double)ng3 / (double)plan->geo.np3;
@@ -519,15 +517,14 @@ int cola_ic_2lpt_adjoint(cola_plan* plan, const float* noise, const float* lam_s
       return rc;
   }
   float* lam_mu2 = w.icR[3];
-  if ((rc = fft3d_c2r(n, P, w.icC2, lam_mu2, w.tw_p, 1.0f, st))) return rc;
+  if ((rc = fft3d_c2r(n, P, w.icC2, lam_mu2, w.tw_p, 1.0f, w.err, st))) return rc;
   // the linear density and the diagonal second derivatives psi_ii
   if ((rc = fft3d_r2c(n, P, noise, w.icC0, w.tw_p, st))) return rc;
   if ((rc = launch_ic_filter(n, P, box, plan->pk_amp, plan->cfg.cosmo.n_s, plan->cfg.cosmo.omega_m,
                              plan->cfg.cosmo.h, w.icC0, st)))
     return rc;
   for (int i = 0; i < 3; ++i) {
-    if ((rc = launch_kmul(n, P, box, 1, i, i, norm, w.icC0, w.icC1, st))) return rc;
-    if ((rc = fft3d_c2r(n, P, w.icC1, w.icR[i], w.tw_p, 1.0f, st))) return rc;
+    if ((rc = fft3d_c2r_factor(n, P, box, 1, i, i, norm, w.icC0, w.icC1, w.icR[i], false, w.tw_p, w.err, st))) return rc;
   }
   // lam_delta_k = sum_ij M_ij FFT(lam_psi_ij) + sum_j (-i k_j / k^2) FFT(lam_s1_j)
   float* tmp = w.icR[4];
@@ -539,8 +536,8 @@ int cola_ic_2lpt_adjoint(cola_plan* plan, const float* noise, const float* lam_s
   }
   const int pairs[3][2] = {{0, 1}, {0, 2}, {1, 2}};
   for (auto& ij : pairs) {  // lam_psi_ij = -2 lam_mu2 psi_ij
-    if ((rc = launch_kmul(n, P, box, 1, ij[0], ij[1], norm, w.icC0, w.icC1, st))) return rc;
-    if ((rc = fft3d_c2r(n, P, w.icC1, tmp, w.tw_p, 1.0f, st))) return rc;
+    if ((rc = fft3d_c2r_factor(n, P, box, 1, ij[0], ij[1], norm, w.icC0, w.icC1, tmp, false, w.tw_p, w.err, st)))
+      return rc;
     if ((rc = launch_ic_adjoint_product(n3, lam_mu2, tmp, nullptr, tmp, st))) return rc;
     if ((rc = fft3d_r2c(n, P, tmp, w.icC1, w.tw_p, st))) return rc;
     if ((rc = launch_kmul_acc(n, P, box, 1, ij[0], ij[1], 1.0f, 1, w.icC1, w.icC2, st))) return rc;
@@ -553,7 +550,7 @@ int cola_ic_2lpt_adjoint(cola_plan* plan, const float* noise, const float* lam_s
   if ((rc = launch_ic_filter(n, P, box, plan->pk_amp, plan->cfg.cosmo.n_s, plan->cfg.cosmo.omega_m,
                              plan->cfg.cosmo.h, w.icC2, st)))
     return rc;
-  return fft3d_c2r(n, P, w.icC2, grad_noise, w.tw_p, norm, st);
+  return fft3d_c2r(n, P, w.icC2, grad_noise, w.tw_p, norm, w.err, st);
 }
 
 int cola_profile(cola_plan* plan, int32_t enable) {

@@ -156,13 +156,16 @@ void twiddle_table(int n, std::vector<float2>& out);
 // ---- launchers (kernels_*.cu) ------------------------------------------------------------
 // FFT passes (fft_kernels.cu)
 int launch_fft_x_r2c(int n, const float* in, float2* out, int64_t nrows, int P, const float2* tw, cudaStream_t st);
-int launch_fft_x_c2r(int n, const float2* in, float* out, int64_t nrows, int P, const float2* tw, float scale,
-                     cudaStream_t st);
 // in place over a half spectrum [n][n][P], along y or along z
 int launch_fft_cols(int n, bool inverse, bool along_z, float2* data, int P, const float2* tw, cudaStream_t st);
 // 3-D helpers built on the passes: r2c (x then y then z) and c2r (z, y, x), layout [n][n][P]
 int fft3d_r2c(int n, int P, const float* in, float2* out, const float2* tw, cudaStream_t st);
-int fft3d_c2r(int n, int P, float2* in_destroyed, float* out, const float2* tw, float scale, cudaStream_t st);
+// (err: latches a timeout of the x pass's bulk copies)
+int fft3d_c2r(int n, int P, float2* in_destroyed, float* out, const float2* tw, float scale, int* err, cudaStream_t st);
+// c2r of a spectral factor (kinds of SpectralFactor, fft_kernels.cu) times `in`, through tmp; with
+// sub_sq out loses the squares of the result instead of receiving it
+int fft3d_c2r_factor(int n, int P, double box, int kind, int i, int j, float factor_scale, const float2* in,
+                     float2* tmp, float* out, bool sub_sq, const float2* tw, int* err, cudaStream_t st);
 
 // PM kernels (pm_kernels.cu)
 int launch_keys(const Geometry& g, const Tiles& t, const float* s, int* keys, int* counts, int* err, cudaStream_t st);
@@ -209,12 +212,8 @@ int launch_kick_drift4(const Geometry& g, const float4* f4, float* s, float* v, 
 int launch_noise(int np, uint64_t seed, float* out, cudaStream_t st);
 int launch_ic_filter(int np, int P, double box, double amp, double n_s, double omega_m, double h, float2* wk,
                      cudaStream_t st);
-// out = factor(k) * in on the half spectrum; kind selects the operator (see ic_kernels.cu)
-int launch_kmul(int n, int P, double box, int kind, int i, int j, float scale, const float2* in, float2* out,
-                cudaStream_t st);
 int launch_source_2lpt(int64_t n3, const float* fxx, const float* fyy, const float* fzz, float* out_acc,
                        cudaStream_t st);
-int launch_source_sub_sq(int64_t n3, const float* f, float* acc, cudaStream_t st);
 int launch_ic_assemble(int64_t n3, float d1, float d2, float t1, float t2, const float* s1, const float* s2,
                        float* s, float* v, cudaStream_t st);
 

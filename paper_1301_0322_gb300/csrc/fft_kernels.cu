@@ -68,33 +68,101 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * x_rows<N>())
   }
 }
 
-// Half-spectrum rows -> real rows of length N (unscaled inverse, times `scale`).
-template <int N>
-__global__ void __launch_bounds__(FFTConf<N / 2>::T * x_rows<N>())
+// Half-spectrum rows -> real rows of length N (unscaled inverse, times `scale`): the persistent
+// inverse-x pass of the force with one component.  SUB_SQ: the rows are not stored but their
+// squares taken off what out holds (the 2LPT source's cross terms).  256^3: 51 us with one item per
+// block read through registers, 25 this way.
+template <int N, bool SUB_SQ>
+__global__ void __launch_bounds__(FFTConf<N / 2>::T * c2r3_rows<N>(), 3)
     k_fft_x_c2r(const float2* __restrict__ in, float* __restrict__ out, int P, const float2* __restrict__ tw,
-                float scale) {
-  constexpr int M = N / 2, T = FFTConf<M>::T, RB = x_rows<N>(), LD = xrow_ld<M>();
-  constexpr int R0 = first_radix<FFTConf<M>>();
-  extern __shared__ __align__(16) float2 smem[];
-  float2* stab = smem + RB * LD;
-  stw_fill<FFTConf<M>, 2>(stab, tw, threadIdx.x, T * RB);
+                float scale, int* __restrict__ err) {
+  constexpr int M = N / 2, RB = c2r3_rows<N>(), LD = xrow_ld<M>();
+  extern __shared__ __align__(128) float2 smem[];
+  __shared__ __align__(8) uint64_t bars[2];
+  float2* stab = smem + 2 * RB * LD;
+  stw_fill<FFTConf<M>, 2>(stab, tw, threadIdx.x, blockDim.x);
   const SmemTw<FFTConf<M>> stw{stab};
-  const int t = threadIdx.x % T, w = threadIdx.x / T;
-  const int64_t row = (int64_t)blockIdx.x * RB + w;
-  const float2* src = in + row * P;
-  float2* buf = smem + w * LD;
-  for (int k = t; k <= M; k += T) buf[xpad<R0>(k)] = src[k];
-  __syncthreads();
-  auto load = [&](int n) -> float2 {
-    const float2 a = buf[xpad<R0>(n)], b = c_conj(buf[xpad<R0>(M - n)]);
-    const float2 e = c_add(a, b);
-    const float2 o = c_mul(c_sub(a, b), c_conj(__ldg(tw + n)));
-    return make_float2(e.x - o.y, e.y + o.x);  // e + i o
+  c2r_walk<N, RB>(
+      smem, bars, (int64_t)N * N / RB, P, err, [&](int64_t item) { return in + item * RB * P; },
+      [&](int64_t item, float2* rows) {
+        float2* dst = reinterpret_cast<float2*>(out + item * RB * N);
+        c2r_rows<N, RB>(rows, 1, 0.0f, tw, stw, [&](int w, int n, float2 x) {
+          float2* p = dst + w * M + n;
+          const float2 r = c_scale(x, scale);
+          if constexpr (SUB_SQ) {
+            const float2 acc = *p;
+            *p = make_float2(fmaf(-r.x, r.x, acc.x), fmaf(-r.y, r.y, acc.y));
+          } else {
+            *p = r;
+          }
+        });
+      });
+}
+
+// Spectral factor of one mode on its way into the inverse z pass (mode numbers nx, ny, nz):
+//   kind 0: scale * (i k_i) / k^2 * a          (s1_i; with scale < 0: s2 from mu2)
+//   kind 1: scale * (i k_i)(i k_j) / k^2 * a   (psi1_{i,j})
+// first derivatives zero on their Nyquist plane
+struct SpectralFactor {
+  int kind, i, j;
+  float kf, scale;
+};
+template <int N>
+__device__ __forceinline__ float2 spectral_mul(const SpectralFactor& f, int nx, int ny, int nz, float2 a) {
+  const int m2 = nx * nx + ny * ny + nz * nz;
+  if (m2 == 0) return make_float2(0.f, 0.f);
+  const float inv_k2 = f.scale / (f.kf * f.kf * (float)m2);
+  auto k_of = [&](int c) {
+    const int m = c == 0 ? nx : (c == 1 ? ny : nz);
+    return (m == N / 2 || m == -N / 2) ? 0.0f : f.kf * (float)m;
   };
-  auto mem = [&](int n) -> float2& { return buf[xpad<R0>(n)]; };
-  float2* dst = reinterpret_cast<float2*>(out + row * N);
-  auto store = [&](int n, float2 x) { dst[n] = c_scale(x, scale); };
-  fft_1d<M, 2, true>(t, stw, load, mem, store);
+  const float ki = k_of(f.i);
+  if (f.kind == 0) return make_float2(__fmul_rn(__fmul_rn(-ki, a.y), inv_k2), __fmul_rn(__fmul_rn(ki, a.x), inv_k2));
+  const float kk = __fmul_rn(__fmul_rn(-ki, k_of(f.j)), inv_k2);
+  return make_float2(__fmul_rn(kk, a.x), __fmul_rn(kk, a.y));
+}
+
+// The inverse z pass of `factor` times the half spectrum `in`, into `out` (a launch of the factor
+// alone reads and writes the spectrum once more: 42 us at 256^3).
+template <int N>
+__global__ void __launch_bounds__(ColsCfg<N, kColsPlain>::THREADS, ColsCfg<N, kColsPlain>::MIN_BLOCKS)
+    k_fft_z_factor(const float2* __restrict__ in, float2* __restrict__ out, SpectralFactor factor,
+                   const float2* __restrict__ tw) {
+  extern __shared__ __align__(16) float2 smem[];
+  using Cfg = ColsCfg<N, kColsPlain>;
+  using V = typename Cfg::V;
+  float2* stab = smem + Cfg::TABLE;
+  stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
+  __syncthreads();
+  const SmemTw<FFTConf<N>> stw{stab};
+  constexpr int64_t P = half_pitch<N>();
+  constexpr int E = Cfg::C::E, T = Cfg::C::T;
+  cols_walk<Cfg>(in, P, N * P, N, smem, [&](const auto& s, const auto& mem, auto& next) {
+    V u[E];
+    mem.collect(u, in + s.first, s.step(), s.valid);
+    const int ny = signed_mode(s.slab, N);
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const int nz = signed_mode(mem.t + T * m, N);
+      if constexpr (Cfg::K == 1) {
+        u[m] = spectral_mul<N>(factor, s.kx, ny, nz, u[m]);
+      } else {
+        const float2 a = spectral_mul<N>(factor, s.kx, ny, nz, make_float2(u[m].re.x, u[m].im.x));
+        const float2 b = spectral_mul<N>(factor, s.kx + 1, ny, nz, make_float2(u[m].re.y, u[m].im.y));
+        u[m] = V{make_float2(a.x, b.x), make_float2(a.y, b.y)};
+      }
+    }
+    auto after_reads = [&] {
+      mem.sync();
+      next();
+    };
+    fft_regs<N, 1, true>(u, mem.t, stw, mem, after_reads);
+    if (s.valid) {
+      float2* p = out + s.first;
+#pragma unroll
+      for (int m = 0; m < E; ++m, p += s.step()) c_store(p, u[m]);
+    }
+  });
 }
 
 // persistent per-size kernel labels for the profiler
@@ -125,14 +193,48 @@ static int x_r2c(const float* in, float2* out, int64_t nrows, int P, const float
   return COLA_OK;
 }
 
+template <int N, bool SUB_SQ>
+static int x_c2r_t(const float2* in, float* out, int P, const float2* tw, float scale, int* err, cudaStream_t st) {
+  constexpr int M = N / 2, RB = c2r3_rows<N>(), NT = FFTConf<M>::T * RB;
+  constexpr size_t smem = (size_t)(2 * RB * xrow_ld<M>() + stw_size<FFTConf<M>>()) * sizeof(float2);
+  static_assert((N * N) % RB == 0, "whole items");
+  if (P % 4) return fail(COLA_EINVAL, "fft x pass: row pitch must be a multiple of 4 complex");
+  static std::atomic<int> resident[64] = {};
+  int dev = 0;
+  COLA_CUDA_CHECK(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return fail(COLA_EUNSUPPORTED, "device index above 63");
+  int cap = resident[dev].load(std::memory_order_acquire);
+  if (!cap) {
+    int occ = 0, sms = 0;
+    allow_smem(k_fft_x_c2r<N, SUB_SQ>, smem);
+    COLA_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fft_x_c2r<N, SUB_SQ>, NT, smem));
+    COLA_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (occ < 1) return fail(COLA_EUNSUPPORTED, "inverse x pass does not fit on an SM");
+    cap = occ * sms;
+    resident[dev].store(cap, std::memory_order_release);
+  }
+  const unsigned grid = (unsigned)std::min<int64_t>((int64_t)N * N / RB, cap);
+  LaunchScope ls_(label<N>("c2r"), st);
+  k_fft_x_c2r<N, SUB_SQ><<<grid, NT, smem, st>>>(in, out, P, tw, scale, err);
+  COLA_LAUNCH_CHECK();
+  return COLA_OK;
+}
 template <int N>
-static int x_c2r(const float2* in, float* out, int64_t nrows, int P, const float2* tw, float scale, cudaStream_t st) {
-  constexpr int M = N / 2, RB = x_rows<N>();
-  const size_t smem = (size_t)(RB * xrow_ld<M>() + stw_size<FFTConf<M>>()) * sizeof(float2);
-  if (nrows % RB) return fail(COLA_EINVAL, "fft x pass: row count not a multiple of the block rows");
-  allow_smem(k_fft_x_c2r<N>, smem);
-  { LaunchScope ls_(label<N>("c2r"), st);
-  k_fft_x_c2r<N><<<(unsigned)(nrows / RB), FFTConf<M>::T * RB, smem, st>>>(in, out, P, tw, scale); }
+static int x_c2r(const float2* in, float* out, int P, const float2* tw, float scale, bool sub_sq, int* err,
+                 cudaStream_t st) {
+  return sub_sq ? x_c2r_t<N, true>(in, out, P, tw, scale, err, st) : x_c2r_t<N, false>(in, out, P, tw, scale, err, st);
+}
+
+template <int N>
+static int z_factor(const float2* in, float2* out, int P, const SpectralFactor& factor, const float2* tw,
+                    cudaStream_t st) {
+  if (P != half_pitch<N>()) return fail(COLA_EINVAL, "fft column pass: unexpected row pitch");
+  using Cfg = ColsCfg<N, kColsPlain>;
+  constexpr size_t smem = cols_smem<Cfg>(0);
+  unsigned grid = 0;
+  if (const int rc = cols_grid<Cfg, k_fft_z_factor<N>>(smem, Cfg::STRIPS * N, &grid)) return rc;
+  LaunchScope ls_(label<N>("inv"), st);
+  k_fft_z_factor<N><<<grid, Cfg::THREADS, smem, st>>>(in, out, factor, tw);
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
@@ -181,12 +283,26 @@ int launch_fft_x_r2c(int n, const float* in, float2* out, int64_t nrows, int P, 
   }
 }
 
-int launch_fft_x_c2r(int n, const float2* in, float* out, int64_t nrows, int P, const float2* tw, float scale,
+int launch_fft_x_c2r(int n, const float2* in, float* out, int P, const float2* tw, float scale, bool sub_sq, int* err,
                      cudaStream_t st) {
   switch (n) {
 #define X(N) \
   case N:    \
-    return x_c2r<N>(in, out, nrows, P, tw, scale, st);
+    return x_c2r<N>(in, out, P, tw, scale, sub_sq, err, st);
+    COLA_FOR_SIZES(X)
+#undef X
+    default:
+      return fail(COLA_EUNSUPPORTED, "fft: unsupported length " + std::to_string(n));
+  }
+}
+
+int launch_fft_z_factor(int n, int P, double box, int kind, int i, int j, float scale, const float2* in, float2* out,
+                        const float2* tw, cudaStream_t st) {
+  const SpectralFactor factor{kind, i, j, (float)(2.0 * 3.14159265358979323846 / box), scale};
+  switch (n) {
+#define X(N) \
+  case N:    \
+    return z_factor<N>(in, out, P, factor, tw, st);
     COLA_FOR_SIZES(X)
 #undef X
     default:
@@ -215,13 +331,21 @@ int fft3d_r2c(int n, int P, const float* in, float2* out, const float2* tw, cuda
   return launch_fft_cols(n, false, true, out, P, tw, st);
 }
 
-int fft3d_c2r(int n, int P, float2* in, float* out, const float2* tw, float scale, cudaStream_t st) {
-  const int64_t nn = n;
+int fft3d_c2r(int n, int P, float2* in, float* out, const float2* tw, float scale, int* err, cudaStream_t st) {
   int rc = launch_fft_cols(n, true, true, in, P, tw, st);
   if (rc) return rc;
   rc = launch_fft_cols(n, true, false, in, P, tw, st);
   if (rc) return rc;
-  return launch_fft_x_c2r(n, in, out, nn * nn, P, tw, scale, st);
+  return launch_fft_x_c2r(n, in, out, P, tw, scale, false, err, st);
+}
+
+int fft3d_c2r_factor(int n, int P, double box, int kind, int i, int j, float factor_scale, const float2* in,
+                     float2* tmp, float* out, bool sub_sq, const float2* tw, int* err, cudaStream_t st) {
+  int rc = launch_fft_z_factor(n, P, box, kind, i, j, factor_scale, in, tmp, tw, st);
+  if (rc) return rc;
+  rc = launch_fft_cols(n, true, false, tmp, P, tw, st);
+  if (rc) return rc;
+  return launch_fft_x_c2r(n, tmp, out, P, tw, 1.0f, sub_sq, err, st);
 }
 
 }  // namespace cola

@@ -91,50 +91,12 @@ __global__ void k_ic_filter(int n, int P, float kf, float amp_scale, float n_s, 
   }
 }
 
-// First derivative factor i k_j, zero on the Nyquist plane |n_j| = n/2.
-__device__ __forceinline__ float kcomp(const Mode& m, int j, int n, float kf) {
-  const int c = j == 0 ? m.nx : (j == 1 ? m.ny : m.nz);
-  return (c == n / 2 || c == -n / 2) ? 0.0f : kf * (float)c;
-}
-
-// kind 0: out = scale * (i k_i) / k^2 * in                (s1_i; with scale < 0: s2 from mu2)
-// kind 1: out = scale * (i k_i)(i k_j) / k^2 * in         (psi1_{i,j})
-__global__ void k_kmul(int n, int P, float kf, int kind, int i_, int j_, float scale, const float2* __restrict__ in,
-                       float2* __restrict__ out) {
-  const int64_t total = (int64_t)n * n * (n / 2 + 1);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const Mode m = mode_of(i, n, P);
-    const int m2 = m.nx * m.nx + m.ny * m.ny + m.nz * m.nz;
-    float2 r = make_float2(0.f, 0.f);
-    if (m2 != 0) {
-      const float inv_k2 = scale / (kf * kf * (float)m2);
-      const float2 a = in[m.off];
-      const float ki = kcomp(m, i_, n, kf);
-      if (kind == 0) {  // i ki a / k^2
-        r = make_float2(-ki * a.y * inv_k2, ki * a.x * inv_k2);
-      } else {  // -ki kj a / k^2
-        const float kk = -ki * kcomp(m, j_, n, kf) * inv_k2;
-        r = make_float2(kk * a.x, kk * a.y);
-      }
-    }
-    out[m.off] = r;
-  }
-}
-
 // acc = fxx fyy + fxx fzz + fyy fzz  (diagonal part of mu2)
 __global__ void k_source_diag(int64_t n3, const float* __restrict__ fxx, const float* __restrict__ fyy,
                               const float* __restrict__ fzz, float* __restrict__ acc) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x) {
     const float a = fxx[i], b = fyy[i], c = fzz[i];
     acc[i] = a * b + a * c + b * c;
-  }
-}
-
-// acc -= f^2  (off-diagonal part of mu2)
-__global__ void k_source_sub_sq(int64_t n3, const float* __restrict__ f, float* __restrict__ acc) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x) {
-    const float x = f[i];
-    acc[i] = fmaf(-x, x, acc[i]);
   }
 }
 
@@ -177,27 +139,10 @@ int launch_ic_filter(int np, int P, double box, double amp, double n_s, double o
   return COLA_OK;
 }
 
-int launch_kmul(int n, int P, double box, int kind, int i, int j, float scale, const float2* in, float2* out,
-                cudaStream_t st) {
-  const float kf = (float)(2.0 * 3.14159265358979323846 / box);
-  const int64_t total = (int64_t)n * n * (n / 2 + 1);
-  { LaunchScope ls_("kmul", st);
-  k_kmul<<<grid_for(total), 256, 0, st>>>(n, P, kf, kind, i, j, scale, in, out); }
-  COLA_LAUNCH_CHECK();
-  return COLA_OK;
-}
-
 int launch_source_2lpt(int64_t n3, const float* fxx, const float* fyy, const float* fzz, float* out_acc,
                        cudaStream_t st) {
   { LaunchScope ls_("source_diag", st);
   k_source_diag<<<grid_for(n3), 256, 0, st>>>(n3, fxx, fyy, fzz, out_acc); }
-  COLA_LAUNCH_CHECK();
-  return COLA_OK;
-}
-
-int launch_source_sub_sq(int64_t n3, const float* f, float* acc, cudaStream_t st) {
-  { LaunchScope ls_("source_sub_sq", st);
-  k_source_sub_sq<<<grid_for(n3), 256, 0, st>>>(n3, f, acc); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }

@@ -563,9 +563,10 @@ __device__ __forceinline__ void c2r3_issue(float2* stage, const float2* src_rows
 
 // Inverse x transform of the staged rows into F rows (pitch N floats); comp 0 applies i k_x.
 // tw: the base twiddle table; stw: the stage twiddles (the base table or an SmemTw table)
-template <int N, int RB, class CM = FFTConf<N / 2>, class STW>
-__device__ __forceinline__ void c2r3_compute(float2* stage, float* __restrict__ Frows, int comp, float kf,
-                                             const float2* __restrict__ tw, const STW& stw) {
+// (put(w, n, x): element n of row w, two real values)
+template <int N, int RB, class CM = FFTConf<N / 2>, class STW, class Put>
+__device__ __forceinline__ void c2r_rows(float2* stage, int comp, float kf, const float2* __restrict__ tw,
+                                         const STW& stw, Put&& put) {
   constexpr int M = N / 2, T = CM::T, LD = xrow_ld<M>(), R0 = first_radix<CM>();
   static_assert(T * RB <= 1024, "block too large");
   const int t = threadIdx.x % T, w = threadIdx.x / T;
@@ -581,14 +582,48 @@ __device__ __forceinline__ void c2r3_compute(float2* stage, float* __restrict__ 
     return make_float2(__fsub_rn(e.x, o.y), __fadd_rn(e.y, o.x));
   };
   auto mem = [&](int n) -> float2& { return buf[xpad<R0>(n)]; };
-  float2* dst = reinterpret_cast<float2*>(Frows + (int64_t)w * N);
-  auto store = [&](int n, float2 x) { dst[n] = x; };
+  auto store = [&](int n, float2 x) { put(w, n, x); };
   fft_1d<M, 2, true, CM>(t, stw, load, mem, store);
 }
-template <int N, int RB, class CM = FFTConf<N / 2>>
+template <int N, int RB, class CM = FFTConf<N / 2>, class STW>
 __device__ __forceinline__ void c2r3_compute(float2* stage, float* __restrict__ Frows, int comp, float kf,
-                                             const float2* __restrict__ tw) {
-  c2r3_compute<N, RB, CM>(stage, Frows, comp, kf, tw, tw);
+                                             const float2* __restrict__ tw, const STW& stw) {
+  c2r_rows<N, RB, CM>(stage, comp, kf, tw, stw,
+                      [&](int w, int n, float2 x) { reinterpret_cast<float2*>(Frows + (int64_t)w * N)[n] = x; });
+}
+
+// The persistent inverse-x loop over `total` items of RB rows: the rows of item i at src_of(i),
+// its transform done by one(item, staged rows).  Each block walks items blockIdx.x, blockIdx.x +
+// gridDim.x, ... with the bulk copy of its next item in flight (two buffers at `stages`).
+template <int N, int RB, class Src, class One>
+__device__ __forceinline__ void c2r_walk(float2* stages, uint64_t (&bars)[2], int64_t total, int P,
+                                         int* __restrict__ err, Src&& src_of, One&& one) {
+  constexpr int LD = xrow_ld<N / 2>();
+  if (threadIdx.x == 0) {
+    mbar_init(&bars[0], 1);
+    mbar_init(&bars[1], 1);
+    mbar_fence_init();
+  }
+  __syncthreads();
+  int64_t item = blockIdx.x;
+  if (item < total && threadIdx.x < 32) c2r3_issue(stages, src_of(item), RB, P, LD, &bars[0]);
+  for (int it = 0; item < total; ++it, item += gridDim.x) {
+    const int b = it & 1;
+    const int64_t ahead = item + gridDim.x;
+    // (the other buffer was consumed at iteration it - 1, free after its closing barrier)
+    if (ahead < total && threadIdx.x < 32) c2r3_issue(stages + (b ^ 1) * RB * LD, src_of(ahead), RB, P, LD, &bars[b ^ 1]);
+    const bool ok = mbar_wait(&bars[b], (it >> 1) & 1);
+    if (__syncthreads_or(!ok)) {
+      // leave no bulk copy in flight into shared memory the block releases: wait again (bounded)
+      // for the copy that timed out and for the later one if it was issued
+      if (threadIdx.x == 0) atomicOr(err, kErrTimeout);
+      mbar_wait(&bars[b], (it >> 1) & 1);
+      if (ahead < total) mbar_wait(&bars[b ^ 1], ((it + 1) >> 1) & 1);
+      return;
+    }
+    one(item, stages + b * RB * LD);
+    __syncthreads();
+  }
 }
 
 }  // namespace cola

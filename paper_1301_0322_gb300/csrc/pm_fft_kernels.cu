@@ -107,13 +107,6 @@ __global__ void __launch_bounds__(ColsCfg<N, kColsY>::THREADS, ColsCfg<N, kColsY
   park.close();
 }
 
-// Persistent: each block walks items blockIdx.x, blockIdx.x + gridDim.x, ... with the bulk
-// copies of its next NB - 1 items in flight during the transform of the current one (NB buffers).
-template <int N>
-__host__ __device__ constexpr int c2r3_stages() {
-  return 2;
-}
-
 // resident blocks per SM of the inverse-x pass: four at N = 2048 (128 registers, no spills;
 // 16 warps to cover the shared-memory latency of the staged rows), three otherwise
 template <int N>
@@ -125,49 +118,26 @@ template <int N>
 __global__ void __launch_bounds__(FFTConf<N / 2>::T * c2r3_rows<N>(), c2r3_min_blocks<N>())
     k_fft_x_c2r3(const float2* __restrict__ C, const float2* __restrict__ Gy, const float2* __restrict__ Gz,
                  float* __restrict__ F, int P, float kf, const float2* __restrict__ tw, int* __restrict__ err) {
-  constexpr int M = N / 2, RB = c2r3_rows<N>(), LD = xrow_ld<M>(), NB = c2r3_stages<N>();
+  constexpr int M = N / 2, RB = c2r3_rows<N>(), LD = xrow_ld<M>();
   extern __shared__ __align__(128) float2 c2r_stage[];
-  __shared__ __align__(8) uint64_t bars[NB];
-  const int64_t nrb = (int64_t)N * N / RB, total = 3 * nrb;
-  auto src_of = [&](int64_t item) -> const float2* {
-    const int comp = (int)(item / nrb);
-    const float2* m = comp == 0 ? C : (comp == 1 ? Gy : Gz);
-    return m + (item - comp * nrb) * RB * P;
-  };
+  __shared__ __align__(8) uint64_t bars[2];
+  const int64_t nrb = (int64_t)N * N / RB;
   // stage twiddles, copied once per block (persistent) behind the staging buffers
-  float2* stab = c2r_stage + NB * RB * LD;
+  float2* stab = c2r_stage + 2 * RB * LD;
   stw_fill<FFTConf<M>, 2>(stab, tw, threadIdx.x, blockDim.x);
   const SmemTw<FFTConf<M>> stw{stab};
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < NB; ++k) mbar_init(&bars[k], 1);
-    mbar_fence_init();
-  }
-  __syncthreads();
-  // prologue: the first NB - 1 items
-  for (int k = 0; k < NB - 1; ++k) {
-    const int64_t item = blockIdx.x + (int64_t)k * gridDim.x;
-    if (item < total && threadIdx.x < 32) c2r3_issue(c2r_stage + k * RB * LD, src_of(item), RB, P, LD, &bars[k]);
-  }
-  int64_t item = blockIdx.x;
-  for (int it = 0; item < total; ++it, item += gridDim.x) {
-    const int b = it % NB;
-    const int64_t ahead = item + (int64_t)(NB - 1) * gridDim.x;
-    const int ba = (it + NB - 1) % NB;  // consumed at iteration it - 1, free after its closing barrier
-    if (ahead < total && threadIdx.x < 32) c2r3_issue(c2r_stage + ba * RB * LD, src_of(ahead), RB, P, LD, &bars[ba]);
-    const bool ok = mbar_wait(&bars[b], (it / NB) & 1);
-    if (__syncthreads_or(!ok)) {
-      // leave no bulk copy in flight into shared memory the block releases: wait again (bounded)
-      // for the copy that timed out and for every later one already issued
-      if (threadIdx.x == 0) atomicOr(err, kErrTimeout);
-      for (int k = 0; k < NB; ++k)
-        if (item + (int64_t)k * gridDim.x < total) mbar_wait(&bars[(it + k) % NB], ((it + k) / NB) & 1);
-      return;
-    }
-    const int comp = (int)(item / nrb);
-    const int64_t row0 = (item - comp * nrb) * RB;
-    c2r3_compute<N, RB>(c2r_stage + b * RB * LD, F + (int64_t)comp * N * N * N + row0 * N, comp, kf, tw, stw);
-    __syncthreads();
-  }
+  c2r_walk<N, RB>(
+      c2r_stage, bars, 3 * nrb, P, err,
+      [&](int64_t item) -> const float2* {
+        const int comp = (int)(item / nrb);
+        const float2* m = comp == 0 ? C : (comp == 1 ? Gy : Gz);
+        return m + (item - comp * nrb) * RB * P;
+      },
+      [&](int64_t item, float2* rows) {
+        const int comp = (int)(item / nrb);
+        const int64_t row0 = (item - comp * nrb) * RB;
+        c2r3_compute<N, RB>(rows, F + (int64_t)comp * N * N * N + row0 * N, comp, kf, tw, stw);
+      });
 }
 
 // ---- launchers ---------------------------------------------------------------------------------------------------
@@ -248,7 +218,7 @@ static int force_passes_t(const Geometry& g, const Tiles& tl, const uint4* rec, 
   // 5. inverse x passes (persistent, bulk-copy pipelined)
   {
     constexpr int RB = c2r3_rows<N>(), T = FFTConf<M>::T;
-    const size_t smem = sizeof(float2) * (c2r3_stages<N>() * RB * xrow_ld<M>() + stw_size<FFTConf<M>>());
+    const size_t smem = sizeof(float2) * (2 * RB * xrow_ld<M>() + stw_size<FFTConf<M>>());
     if ((rc = set_smem(k_fft_x_c2r3<N>, smem))) return rc;
     const int64_t nrows = (int64_t)N * N;
     if (nrows % RB) return fail(COLA_EINVAL, "fused c2r: row count not a multiple of the block rows");
