@@ -174,7 +174,7 @@ def algorithmic_bytes(name, n_p, ng):
 
 # the sources the force-evaluation kernels are compiled from (their measured DRAM traffic stays
 # valid while these are unchanged)
-FORCE_SOURCES = ("cola_internal.cuh", "cols_launch.cuh", "fft.cuh", "fft_kernels.cu", "particle_bodies.cuh",
+FORCE_SOURCES = ("cola_internal.cuh", "cols_launch.cuh", "fft.cuh", "fft_kernels.cu", "launch.cuh", "particle_bodies.cuh",
                  "pm_bodies.cuh", "pm_common.cuh", "pm_fft_kernels.cu", "pm_kernels.cu", "tma.cuh", "tmem.cuh")
 
 

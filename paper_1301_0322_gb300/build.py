@@ -15,7 +15,7 @@ SOURCES = ["api.cu", "coeffs.cpp", "fft_kernels.cu", "pm_kernels.cu", "ic_kernel
            "power_noalloc.cu", "pm_fft_kernels.cu", "adjoint_kernels.cu", "ensemble.cu",
            "fof.cu"]
 HEADERS = ["cola_internal.cuh", "fft.cuh", "pm_common.cuh", "profiler.cuh", "pm_bodies.cuh", "particle_bodies.cuh",
-           "tma.cuh", "tmem.cuh", "cols_launch.cuh"]
+           "tma.cuh", "tmem.cuh", "cols_launch.cuh", "launch.cuh"]
 NVCC = os.environ.get("NVCC", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC"] + ARCH

@@ -11,6 +11,7 @@ namespace cola {
 static thread_local std::string g_last_error;
 std::atomic<unsigned long long> g_launches{0};
 thread_local Profiler* t_profiler = nullptr;
+thread_local bool t_overlap = false;
 
 void set_error(const std::string& msg) { g_last_error = msg; }
 
@@ -68,6 +69,11 @@ static int check_ws(const cola_plan* p) {
   return COLA_OK;
 }
 
+// Launches overlap (launch.cuh) up to 256 cells or particles per side, where the gaps between them
+// count.  Beyond, they lose: blocks of the next kernel that sit on an SM early keep it at the
+// running kernel's split of shared memory and L1 (one step 256^3/768^3 9.22 ms, 10.96 overlapped).
+static bool small_mesh(int n) { return n <= 256; }
+
 static int padded_half(int n) { return ((n / 2 + 1) + 3) / 4 * 4; }
 
 // particle binning for positions s: keys -> counts -> offsets -> bin-ordered records
@@ -75,7 +81,7 @@ static int bin_particles(cola_plan* p, const float* s, cudaStream_t st) {
   Workspace& w = p->ws;
   int rc = launch_keys(p->geo, p->tiles, s, w.keys, w.counts, w.err, st);
   if (rc) return rc;
-  rc = launch_scan(p->tiles, w.counts, w.offsets, w.cursor, w.scan_blocks, st);
+  rc = launch_scan(p->tiles, w.counts, w.offsets, w.cursor, w.scan_blocks, !p->in_ensemble, st);
   if (rc) return rc;
   return launch_scatter(p->geo, s, w.keys, w.cursor, w.rec, st);
 }
@@ -274,14 +280,14 @@ int cola_coeffs(const cola_plan* plan, double* table) {
 
 int cola_noise(cola_plan* plan, uint64_t seed, float* noise, cola_stream stream) {
   if (!plan || !noise) return fail(COLA_EINVAL, "null argument");
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.np));
   return launch_noise(plan->geo.np, seed, noise, (cudaStream_t)stream);
 }
 
 int cola_ic_2lpt(cola_plan* plan, const float* noise, float* s, float* v, float* s1, float* s2, cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.np));
   if (!noise || !s || !v || !s1 || !s2) return fail(COLA_EINVAL, "null array");
   cudaStream_t st = (cudaStream_t)stream;
   Workspace& w = plan->ws;
@@ -328,7 +334,7 @@ int cola_step(cola_plan* plan, int32_t step, float* s, float* v, const float* s1
               cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.ng));
   if (!s || !v || !s1 || !s2) return fail(COLA_EINVAL, "null array");
   if (step < 0 || step > plan->cfg.nsteps) return fail(COLA_EINVAL, "step out of range");
   cudaStream_t st = (cudaStream_t)stream;
@@ -353,7 +359,7 @@ int cola_step(cola_plan* plan, int32_t step, float* s, float* v, const float* s1
 int cola_force(cola_plan* plan, const float* s, float* g, cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.ng));
   if (!s || !g) return fail(COLA_EINVAL, "null array");
   cudaStream_t st = (cudaStream_t)stream;
   if ((rc = force_meshes(plan, s, st))) return rc;
@@ -364,7 +370,7 @@ int cola_force(cola_plan* plan, const float* s, float* g, cola_stream stream) {
 int cola_density(cola_plan* plan, const float* s, int64_t* rho_fix, float* delta, cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.ng));
   if (!s || (!rho_fix && !delta)) return fail(COLA_EINVAL, "null array");
   cudaStream_t st = (cudaStream_t)stream;
   if ((rc = bin_particles(plan, s, st))) return rc;
@@ -375,7 +381,7 @@ int cola_power(cola_plan* plan, const float* delta, int32_t nbins, double* k, do
                cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.ng));
   if (!delta || !k || !pk || !nmodes) return fail(COLA_EINVAL, "null array");
   if (nbins < 1 || nbins > plan->geo.ng) return fail(COLA_EINVAL, "nbins must be in [1, ng]");
   cudaStream_t st = (cudaStream_t)stream;
@@ -389,7 +395,7 @@ int cola_density_power(cola_plan* plan, const float* s, int32_t nbins, double* k
                        cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.ng));
   if (!s || !k || !pk || !nmodes) return fail(COLA_EINVAL, "null array");
   if (nbins < 1 || nbins > plan->geo.ng) return fail(COLA_EINVAL, "nbins must be in [1, ng]");
   cudaStream_t st = (cudaStream_t)stream;
@@ -406,7 +412,7 @@ int cola_cross_power(cola_plan* plan, const float* delta_a, const float* delta_b
                      cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.ng));
   if (!delta_a || !delta_b || !k || !pk_a || !pk_b || !pk_ab || !rho || !nmax || !nmodes)
     return fail(COLA_EINVAL, "null array");
   if (nbins < 1 || nbins > plan->geo.ng) return fail(COLA_EINVAL, "nbins must be in [1, ng]");
@@ -422,7 +428,7 @@ int cola_cross_power(cola_plan* plan, const float* delta_a, const float* delta_b
 int cola_fft_r2c(cola_plan* plan, int32_t which, const float* in, float* out, cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(which == 0 ? plan->geo.ng : plan->geo.np));
   if (!in || !out) return fail(COLA_EINVAL, "null array");
   if (which != 0 && which != 1) return fail(COLA_EINVAL, "which must be 0 (mesh) or 1 (lattice)");
   cudaStream_t st = (cudaStream_t)stream;
@@ -453,7 +459,7 @@ int cola_step_adjoint(cola_plan* plan, int32_t step, const float* s_ckpt, float*
                       float* lam_s2, cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.ng));
   if (!plan->cfg.adjoint) return fail(COLA_EINVAL, "plan was created without adjoint buffers (cola_config.adjoint)");
   if (!s_ckpt || !lam_s || !lam_v || !lam_s1 || !lam_s2) return fail(COLA_EINVAL, "null array");
   if (step < 0 || step > plan->cfg.nsteps) return fail(COLA_EINVAL, "step out of range");
@@ -499,7 +505,7 @@ int cola_ic_2lpt_adjoint(cola_plan* plan, const float* noise, const float* lam_s
                          float* grad_noise, cola_stream stream) {
   int rc = check_ws(plan);
   if (rc) return rc;
-  ProfilerGuard pg(&plan->prof);
+  ProfilerGuard pg(&plan->prof, small_mesh(plan->geo.np));
   if (!noise || !lam_s || !lam_s1 || !lam_s2 || !grad_noise) return fail(COLA_EINVAL, "null array");
   cudaStream_t st = (cudaStream_t)stream;
   Workspace& w = plan->ws;

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/cola.h"
+#include "launch.cuh"
 #include "profiler.cuh"
 
 namespace cola {
@@ -39,7 +40,7 @@ struct Geometry {
   // division of a 32-bit index by np as a multiply-high and shifts (set_np_divider)
   uint32_t np_mul;
   int np_sh1, np_sh2;
-  // fixed_axis may take its 32-bit path: ratio != 0 and 2^22 <= ng 2^F <= 2^30
+  // fixed_axis may take its 32-bit path: 2^22 <= ng 2^F <= 2^30
   int fast32;
 };
 
@@ -54,7 +55,7 @@ inline void set_np_divider(Geometry& g) {
   g.np_sh1 = l < 1 ? l : 1;
   g.np_sh2 = l > 1 ? l - 1 : 0;
   const int64_t period = (int64_t)g.ng << g.fbits;
-  g.fast32 = g.ratio != 0 && period >= (1LL << 22) && period <= (1LL << 30);
+  g.fast32 = period >= (1LL << 22) && period <= (1LL << 30);
 }
 
 struct Tiles {
@@ -125,6 +126,8 @@ struct cola_plan {
   // one float4 per particle into the first of them when it holds 16 bytes per particle
   bool binned_gather = false;
   bool binned_gather4 = false;
+  // a box of an ensemble: its steps keep the three scan launches of the ensemble's documented 12
+  bool in_ensemble = false;
   // retry limit of the friends-of-friends union-find (cola_set_fof_union_tries)
   int fof_union_tries = 1 << 20;
   std::vector<double> coef64;
@@ -170,7 +173,9 @@ int fft3d_c2r_factor(int n, int P, double box, int kind, int i, int j, float fac
 // PM kernels (pm_kernels.cu)
 int launch_keys(const Geometry& g, const Tiles& t, const float* s, int* keys, int* counts, int* err, cudaStream_t st);
 int scan_block_count(const Tiles& t);
-int launch_scan(const Tiles& t, int* counts, int* offsets, int* cursor, int* block_sums, cudaStream_t st);
+// (one_block: as one launch where the bins are few enough)
+int launch_scan(const Tiles& t, int* counts, int* offsets, int* cursor, int* block_sums, bool one_block,
+                cudaStream_t st);
 int launch_scatter(const Geometry& g, const float* s, const int* keys, int* cursor, uint4* rec,
                    cudaStream_t st);
 int launch_deposit(const Geometry& g, const Tiles& t, const uint4* rec, const int* offsets, int64_t* rho,

@@ -686,7 +686,7 @@ int enqueue_binning(cola_ensemble* e, const float* s, cudaStream_t st) {
   COLA_LAUNCH_CHECK();
   Tiles all{};
   all.nbins = e->total_bins;
-  int rc = launch_scan(all, e->counts, e->offsets, e->cursor, e->scan_blocks, st);
+  int rc = launch_scan(all, e->counts, e->offsets, e->cursor, e->scan_blocks, false, st);
   if (rc) return rc;
   {
     LaunchScope ls_("ens_scatter", st);
@@ -892,6 +892,7 @@ int cola_ensemble_create(const cola_config* boxes, int32_t nbox, cola_ensemble**
       delete e;
       return fail(rc, why);
     }
+    p->in_ensemble = true;
     e->plans.push_back(p);
     e->binned_gather = e->binned_gather && p->binned_gather;
     e->gather_f4 = e->gather_f4 && p->binned_gather4;

@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(ColsCfg<N, kColsPlain>::THREADS, ColsCfg<N, kC
   using Cfg = ColsCfg<N, kColsPlain>;
   float2* stab = smem + Cfg::TABLE;
   stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
+  pdl_begin();
   __syncthreads();
   const SmemTw<FFTConf<N>> stw{stab};
   constexpr int64_t P = half_pitch<N>();
@@ -45,6 +46,7 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * x_rows<N>())
   extern __shared__ __align__(16) float2 smem[];
   float2* stab = smem + RB * LD;
   stw_fill<FFTConf<M>, 2>(stab, tw, threadIdx.x, T * RB);
+  pdl_begin();
   const SmemTw<FFTConf<M>> stw{stab};
   const int t = threadIdx.x % T, w = threadIdx.x / T;
   const int64_t row = (int64_t)blockIdx.x * RB + w;
@@ -82,6 +84,7 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * c2r3_rows<N>(), 3)
   float2* stab = smem + 2 * RB * LD;
   stw_fill<FFTConf<M>, 2>(stab, tw, threadIdx.x, blockDim.x);
   const SmemTw<FFTConf<M>> stw{stab};
+  pdl_begin();
   c2r_walk<N, RB>(
       smem, bars, (int64_t)N * N / RB, P, err, [&](int64_t item) { return in + item * RB * P; },
       [&](int64_t item, float2* rows) {
@@ -133,6 +136,7 @@ __global__ void __launch_bounds__(ColsCfg<N, kColsPlain>::THREADS, ColsCfg<N, kC
   using V = typename Cfg::V;
   float2* stab = smem + Cfg::TABLE;
   stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
+  pdl_begin();
   __syncthreads();
   const SmemTw<FFTConf<N>> stw{stab};
   constexpr int64_t P = half_pitch<N>();
@@ -188,7 +192,7 @@ static int x_r2c(const float* in, float2* out, int64_t nrows, int P, const float
   if (nrows % RB) return fail(COLA_EINVAL, "fft x pass: row count not a multiple of the block rows");
   allow_smem(k_fft_x_r2c<N>, smem);
   { LaunchScope ls_(label<N>("r2c"), st);
-  k_fft_x_r2c<N><<<(unsigned)(nrows / RB), FFTConf<M>::T * RB, smem, st>>>(in, out, P, tw); }
+  launch(k_fft_x_r2c<N>, (unsigned)(nrows / RB), FFTConf<M>::T * RB, smem, st, in, out, P, tw); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
@@ -215,7 +219,7 @@ static int x_c2r_t(const float2* in, float* out, int P, const float2* tw, float 
   }
   const unsigned grid = (unsigned)std::min<int64_t>((int64_t)N * N / RB, cap);
   LaunchScope ls_(label<N>("c2r"), st);
-  k_fft_x_c2r<N, SUB_SQ><<<grid, NT, smem, st>>>(in, out, P, tw, scale, err);
+  launch(k_fft_x_c2r<N, SUB_SQ>, grid, NT, smem, st, in, out, P, tw, scale, err);
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
@@ -234,7 +238,7 @@ static int z_factor(const float2* in, float2* out, int P, const SpectralFactor& 
   unsigned grid = 0;
   if (const int rc = cols_grid<Cfg, k_fft_z_factor<N>>(smem, Cfg::STRIPS * N, &grid)) return rc;
   LaunchScope ls_(label<N>("inv"), st);
-  k_fft_z_factor<N><<<grid, Cfg::THREADS, smem, st>>>(in, out, factor, tw);
+  launch(k_fft_z_factor<N>, grid, Cfg::THREADS, smem, st, in, out, factor, tw);
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
@@ -246,7 +250,7 @@ static int cols_t(float2* data, const float2* tw, cudaStream_t st) {
   unsigned grid = 0;
   if (const int rc = cols_grid<Cfg, k_fft_cols<N, INV, ALONG_Z>>(smem, Cfg::STRIPS * N, &grid)) return rc;
   LaunchScope ls_(label<N>(INV ? "inv" : "fwd"), st);
-  k_fft_cols<N, INV, ALONG_Z><<<grid, Cfg::THREADS, smem, st>>>(data, tw);
+  launch(k_fft_cols<N, INV, ALONG_Z>, grid, Cfg::THREADS, smem, st, data, tw);
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }

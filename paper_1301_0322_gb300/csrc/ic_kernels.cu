@@ -30,6 +30,7 @@ __device__ __forceinline__ void philox4x32_10(uint32_t (&c)[4], uint32_t k0, uin
 // key = (seed lo, seed hi)); uniforms u = ((r >> 8) + 1) 2^-24; Box-Muller pairs (r0, r1) ->
 // cells 4g, 4g+1 (cos, sin) and (r2, r3) -> cells 4g+2, 4g+3.
 __global__ void k_noise(int64_t n3, uint32_t key0, uint32_t key1, float* __restrict__ out) {
+  pdl_begin();
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g * 4 >= n3) return;
   uint32_t c[4] = {(uint32_t)(g & 0xFFFFFFFFll), (uint32_t)(g >> 32), 0u, 0u};
@@ -71,6 +72,7 @@ __device__ __forceinline__ Mode mode_of(int64_t i, int n, int P) {
 
 // delta_k = w_k sqrt(P(k) n^3 / L^3), P = A k^ns T_BBKS(k)^2, k = 0 removed.
 __global__ void k_ic_filter(int n, int P, float kf, float amp_scale, float n_s, float gamma, float2* __restrict__ wk) {
+  pdl_begin();
   const int64_t total = (int64_t)n * n * (n / 2 + 1);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const Mode m = mode_of(i, n, P);
@@ -94,6 +96,7 @@ __global__ void k_ic_filter(int n, int P, float kf, float amp_scale, float n_s, 
 // acc = fxx fyy + fxx fzz + fyy fzz  (diagonal part of mu2)
 __global__ void k_source_diag(int64_t n3, const float* __restrict__ fxx, const float* __restrict__ fyy,
                               const float* __restrict__ fzz, float* __restrict__ acc) {
+  pdl_begin();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x) {
     const float a = fxx[i], b = fyy[i], c = fzz[i];
     acc[i] = a * b + a * c + b * c;
@@ -103,6 +106,7 @@ __global__ void k_source_diag(int64_t n3, const float* __restrict__ fxx, const f
 // s = D1 s1 + D2 s2, v = 0 (2LPT position at a_init; velocity after L-).
 __global__ void k_ic_assemble(int64_t m, float d1, float d2, float t1, float t2, const float* __restrict__ s1,
                               const float* __restrict__ s2, float* __restrict__ s, float* __restrict__ v) {
+  pdl_begin();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     const float a = s1[i], b = s2[i];
     s[i] = fmaf(d1, a, d2 * b);
@@ -120,8 +124,7 @@ int launch_noise(int np, uint64_t seed, float* out, cudaStream_t st) {
   const int64_t groups = (n3 + 3) / 4;
   {
     LaunchScope ls_("noise", st);
-    k_noise<<<(unsigned)((groups + 255) / 256), 256, 0, st>>>(n3, (uint32_t)(seed & 0xFFFFFFFFull),
-                                                              (uint32_t)(seed >> 32), out);
+    launch(k_noise, (unsigned)((groups + 255) / 256), 256, 0, st, n3, (uint32_t)(seed & 0xFFFFFFFFull), (uint32_t)(seed >> 32), out);
   }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
@@ -134,7 +137,7 @@ int launch_ic_filter(int np, int P, double box, double amp, double n_s, double o
   const float amp_scale = (float)std::sqrt(amp * n3 / (box * box * box));
   const int64_t total = (int64_t)np * np * (np / 2 + 1);
   { LaunchScope ls_("ic_filter", st);
-  k_ic_filter<<<grid_for(total), 256, 0, st>>>(np, P, kf, amp_scale, (float)n_s, (float)(omega_m * h), wk); }
+  launch(k_ic_filter, grid_for(total), 256, 0, st, np, P, kf, amp_scale, (float)n_s, (float)(omega_m * h), wk); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
@@ -142,7 +145,7 @@ int launch_ic_filter(int np, int P, double box, double amp, double n_s, double o
 int launch_source_2lpt(int64_t n3, const float* fxx, const float* fyy, const float* fzz, float* out_acc,
                        cudaStream_t st) {
   { LaunchScope ls_("source_diag", st);
-  k_source_diag<<<grid_for(n3), 256, 0, st>>>(n3, fxx, fyy, fzz, out_acc); }
+  launch(k_source_diag, grid_for(n3), 256, 0, st, n3, fxx, fyy, fzz, out_acc); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
@@ -150,7 +153,7 @@ int launch_source_2lpt(int64_t n3, const float* fxx, const float* fyy, const flo
 int launch_ic_assemble(int64_t n3, float d1, float d2, float t1, float t2, const float* s1, const float* s2,
                        float* s, float* v, cudaStream_t st) {
   { LaunchScope ls_("ic_assemble", st);
-  k_ic_assemble<<<grid_for(3 * n3), 256, 0, st>>>(3 * n3, d1, d2, t1, t2, s1, s2, s, v); }
+  launch(k_ic_assemble, grid_for(3 * n3), 256, 0, st, 3 * n3, d1, d2, t1, t2, s1, s2, s, v); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }

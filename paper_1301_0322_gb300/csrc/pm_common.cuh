@@ -4,18 +4,19 @@
 
 namespace cola {
 
+// v / np as a multiply-high and shifts (set_np_divider): integer-pipe instructions only
+__device__ __forceinline__ unsigned div_np(const Geometry& g, unsigned v) {
+  const unsigned t = __umulhi(g.np_mul, v);
+  return (t + ((v - t) >> g.np_sh1)) >> g.np_sh2;
+}
+
 // Lattice index of particle p = (iz np + iy) np + ix.
 __device__ __forceinline__ void lattice_index(const Geometry& g, int64_t p, int& ix, int& iy, int& iz) {
   if (g.np3 <= 0xFFFFFFFFLL) {
-    // quotients by np as multiply-highs (set_np_divider): integer-pipe instructions only
     const unsigned pu = (unsigned)p, n = (unsigned)g.np;
-    auto div_np = [&](unsigned v) -> unsigned {
-      const unsigned t = __umulhi(g.np_mul, v);
-      return (t + ((v - t) >> g.np_sh1)) >> g.np_sh2;
-    };
-    const unsigned r = div_np(pu);
+    const unsigned r = div_np(g, pu);
     ix = (int)(pu - r * n);
-    iz = (int)div_np(r);
+    iz = (int)div_np(g, r);
     iy = (int)(r - (unsigned)iz * n);
   } else {
     const int64_t r = p / g.np;
@@ -38,8 +39,17 @@ __device__ __forceinline__ void fixed_axis(const Geometry& g, int i, float s, in
     // ng 2^F, so f lies in (-2^22, 2^30 + 2^22) and one wrap brings it into [0, ng 2^F).
     // floor(ws) without a conversion instruction: ws + 1.5 2^23 rounded down lies in
     // [2^23, 2^24), where floats are the integers and their bit patterns consecutive.
+    // (where ng is no multiple of np: floor(i ng 2^F / np) = (i ng / np) 2^F + (i ng mod np) 2^F / np,
+    // with i ng < 2^22 and (i ng mod np) 2^F < 2^31; two 64-bit divisions per axis before)
     const int period = g.ng << g.fbits;
-    int f = ((i * g.ratio) << g.fbits) + (__float_as_int(__fadd_rd(ws, 12582912.0f)) - 0x4B400000);
+    int q;
+    if (g.ratio) {
+      q = (i * g.ratio) << g.fbits;
+    } else {
+      const unsigned whole = div_np(g, (unsigned)(i * g.ng)), rest = (unsigned)(i * g.ng) - whole * (unsigned)g.np;
+      q = (int)((whole << g.fbits) + div_np(g, rest << g.fbits));
+    }
+    int f = q + (__float_as_int(__fadd_rd(ws, 12582912.0f)) - 0x4B400000);
     if (f < 0) f += period;
     else if (f >= period) f -= period;
     cell = f >> g.fbits;

@@ -58,9 +58,11 @@ __global__ void __launch_bounds__(deposit_threads<N, TY, TZ>(), deposit_min_bloc
   if constexpr (deposit_table_size<N>() > 0) {
     float2* stab = reinterpret_cast<float2*>(acc + deposit_acc_cells<N, TY, TZ>());
     stw_fill<FFTConf<N / 2>, 2, true>(stab, tw, threadIdx.x, blockDim.x);
+    pdl_begin();
     deposit_fftx_body<N, TY, TZ, FFTConf<N / 2>, deposit_threads<N, TY, TZ>()>(
         g, tl, rec, offsets, out, P, tw, SmemTw<FFTConf<N / 2>, true>{stab}, dscale, err, blockIdx.x, acc, ints);
   } else {
+    pdl_begin();
     deposit_fftx_body<N, TY, TZ, FFTConf<N / 2>, deposit_threads<N, TY, TZ>()>(g, tl, rec, offsets, out, P, tw, tw,
                                                                                dscale, err, blockIdx.x, acc, ints);
   }
@@ -81,7 +83,10 @@ __global__ void __launch_bounds__(ColsCfg<N, kColsZ>::THREADS, ColsCfg<N, kColsZ
   float* sinc2 = reinterpret_cast<float*>(stab + stw_size<FFTConf<N>>());
   stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
   sinc2_fill<N>(sinc2, threadIdx.x, Cfg::THREADS);
-  const ColsPark<Cfg> park(&slot);  // (its block barrier publishes the tables as well)
+  pdl_begin();
+  // (after the wait: a predecessor's blocks must not wait for this kernel's tensor memory; its block
+  // barrier publishes the tables as well)
+  const ColsPark<Cfg> park(&slot);
   const SmemTw<FFTConf<N>> stw{stab};
   cols_walk<Cfg>(A, P, (int64_t)N * P, N, sm, [&](const auto& s, const auto& mem, auto& next) {
     z_green_strip(A, Gz, kf, deconv, norm, stw, sinc2, s, mem, park, next);
@@ -99,6 +104,7 @@ __global__ void __launch_bounds__(ColsCfg<N, kColsY>::THREADS, ColsCfg<N, kColsY
   constexpr int P = half_pitch<N>();
   float2* stab = sm + Cfg::TABLE;
   stw_fill<FFTConf<N>, 1>(stab, tw, threadIdx.x, Cfg::THREADS);
+  pdl_begin();
   const ColsPark<Cfg> park(&slot);
   const SmemTw<FFTConf<N>> stw{stab};
   cols_walk<Cfg>(B, (int64_t)N * P, P, N, sm, [&](const auto& s, const auto& mem, auto& next) {
@@ -126,6 +132,7 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * c2r3_rows<N>(), c2r3_min_b
   float2* stab = c2r_stage + 2 * RB * LD;
   stw_fill<FFTConf<M>, 2>(stab, tw, threadIdx.x, blockDim.x);
   const SmemTw<FFTConf<M>> stw{stab};
+  pdl_begin();
   c2r_walk<N, RB>(
       c2r_stage, bars, 3 * nrb, P, err,
       [&](int64_t item) -> const float2* {
@@ -169,14 +176,12 @@ static int deposit_fftx_t(const Geometry& g, const Tiles& tl, const uint4* rec, 
     const size_t smem = sizeof(unsigned long long) * (deposit_acc_cells<N, 4, 2>() + deposit_table_size<N>());
     if ((rc = set_smem(k_deposit_fftx<N, 4, 2>, smem))) return rc;
     LaunchScope ls_(flabel<N>(0), st);
-    k_deposit_fftx<N, 4, 2><<<tl.nty * tl.ntz, deposit_threads<N, 4, 2>(), smem, st>>>(g, tl, rec, offsets, A, P, tw,
-                                                                                dscale, err);
+    launch(k_deposit_fftx<N, 4, 2>, tl.nty * tl.ntz, deposit_threads<N, 4, 2>(), smem, st, g, tl, rec, offsets, A, P, tw, dscale, err);
   } else if (tl.ty == 2 && tl.tz == 2) {
     const size_t smem = sizeof(unsigned long long) * (deposit_acc_cells<N, 2, 2>() + deposit_table_size<N>());
     if ((rc = set_smem(k_deposit_fftx<N, 2, 2>, smem))) return rc;
     LaunchScope ls_(flabel<N>(0), st);
-    k_deposit_fftx<N, 2, 2><<<tl.nty * tl.ntz, deposit_threads<N, 2, 2>(), smem, st>>>(g, tl, rec, offsets, A, P, tw,
-                                                                                dscale, err);
+    launch(k_deposit_fftx<N, 2, 2>, tl.nty * tl.ntz, deposit_threads<N, 2, 2>(), smem, st, g, tl, rec, offsets, A, P, tw, dscale, err);
   } else {
     return fail(COLA_EUNSUPPORTED, "fused deposit: unsupported tile shape");
   }
@@ -203,7 +208,7 @@ static int force_passes_t(const Geometry& g, const Tiles& tl, const uint4* rec, 
     constexpr size_t smem = cols_smem<Cfg>(N);
     if ((rc = cols_grid<Cfg, k_fft_z_green<N>>(smem, Cfg::STRIPS * N, &grid))) return rc;
     LaunchScope ls_(flabel<N>(1), st);
-    k_fft_z_green<N><<<grid, Cfg::THREADS, smem, st>>>(A, Gz, kf, deconv, norm, tw);
+    launch(k_fft_z_green<N>, grid, Cfg::THREADS, smem, st, A, Gz, kf, deconv, norm, tw);
     COLA_LAUNCH_CHECK();
   }
   // 4. inverse y passes
@@ -212,7 +217,7 @@ static int force_passes_t(const Geometry& g, const Tiles& tl, const uint4* rec, 
     constexpr size_t smem = cols_smem<Cfg>(0);
     if ((rc = cols_grid<Cfg, k_fft_y_inv3<N>>(smem, Cfg::STRIPS * N, &grid))) return rc;
     LaunchScope ls_(flabel<N>(2), st);
-    k_fft_y_inv3<N><<<grid, Cfg::THREADS, smem, st>>>(A, Gy, Gz, kf, tw);
+    launch(k_fft_y_inv3<N>, grid, Cfg::THREADS, smem, st, A, Gy, Gz, kf, tw);
     COLA_LAUNCH_CHECK();
   }
   // 5. inverse x passes (persistent, bulk-copy pipelined)
@@ -238,7 +243,7 @@ static int force_passes_t(const Geometry& g, const Tiles& tl, const uint4* rec, 
     const int64_t items = 3 * nrows / RB;
     const unsigned grid = (unsigned)std::min<int64_t>(items, grid_cap[dev]);
     LaunchScope ls_(flabel<N>(3), st);
-    k_fft_x_c2r3<N><<<grid, T * RB, smem, st>>>(A, Gy, Gz, F, P, kf, tw, err);
+    launch(k_fft_x_c2r3<N>, grid, T * RB, smem, st, A, Gy, Gz, F, P, kf, tw, err);
     COLA_LAUNCH_CHECK();
   }
   return COLA_OK;

@@ -48,6 +48,7 @@ template <int NF>
 __global__ void k_power_bin(int ng, int P, float kf, float pnorm, int nbins, int b0, int b1,
                             const float2* __restrict__ dk, const float2* __restrict__ dk2,
                             double* __restrict__ partial) {
+  pdl_begin();
   constexpr int NQ = NF == 1 ? 3 : 5;
   static_assert(NQ <= kPowerQuantities, "partial sums beyond the sized buffers");
   extern __shared__ double pacc[];
@@ -185,6 +186,7 @@ __device__ __forceinline__ void shell_sums(int nbins, int nblocks, const double*
 __global__ void __launch_bounds__(128) k_power_finish(int nbins, int nblocks, const double* __restrict__ partial,
                                                       double* __restrict__ k, double* __restrict__ pk,
                                                       int64_t* __restrict__ nmodes) {
+  pdl_begin();
   const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (b >= nbins) return;
   double s[3];
@@ -203,6 +205,7 @@ __global__ void __launch_bounds__(128) k_cross_finish(int nbins, int nblocks, co
                                                       double* __restrict__ pb, double* __restrict__ pab,
                                                       double* __restrict__ rho, double* __restrict__ nmax,
                                                       int64_t* __restrict__ nmodes) {
+  pdl_begin();
   const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (b >= nbins) return;
   double s[5];
@@ -221,6 +224,7 @@ __global__ void __launch_bounds__(128) k_cross_finish(int nbins, int nblocks, co
 }
 
 __global__ void k_unpad(int n, int P, const float2* __restrict__ in, float2* __restrict__ out) {
+  pdl_begin();
   const int nh = n / 2 + 1;
   const int64_t total = (int64_t)n * n * nh;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
@@ -260,8 +264,7 @@ static int power_bin_t(int ng, int P, double box, int nbins, const float2* dk, c
     const int b1 = std::min(nbins, b0 + range);
     {
       LaunchScope ls_(NF == 1 ? "power_bin" : "cross_bin", st);
-      k_power_bin<NF><<<kPowerBlocks, 32 * kPowerWarps, smem, st>>>(ng, P, kf, pnorm, nbins, b0, b1, dk, dk2,
-                                                                      partial);
+      launch(k_power_bin<NF>, kPowerBlocks, 32 * kPowerWarps, smem, st, ng, P, kf, pnorm, nbins, b0, b1, dk, dk2, partial);
     }
     COLA_LAUNCH_CHECK();
   }
@@ -281,8 +284,7 @@ int launch_cross_finish(int nbins, const double* partial, double* k, double* pa,
                         double* nmax, int64_t* nmodes, cudaStream_t st) {
   {
     LaunchScope ls_("cross_finish", st);
-    k_cross_finish<<<(nbins + 3) / 4, 128, 0, st>>>(nbins, kPowerBlocks, partial, k, pa, pb, pab, rho, nmax,
-                                                         nmodes);
+    launch(k_cross_finish, (nbins + 3) / 4, 128, 0, st, nbins, kPowerBlocks, partial, k, pa, pb, pab, rho, nmax, nmodes);
   }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
@@ -291,7 +293,7 @@ int launch_cross_finish(int nbins, const double* partial, double* k, double* pa,
 int launch_power_finish(int nbins, const double* partial, double* k, double* pk, int64_t* nmodes, cudaStream_t st) {
   {
     LaunchScope ls_("power_finish", st);
-    k_power_finish<<<(nbins + 3) / 4, 128, 0, st>>>(nbins, kPowerBlocks, partial, k, pk, nmodes);
+    launch(k_power_finish, (nbins + 3) / 4, 128, 0, st, nbins, kPowerBlocks, partial, k, pk, nmodes);
   }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
@@ -301,7 +303,7 @@ int launch_unpad(int n, int P, const float2* in, float2* out, cudaStream_t st) {
   const int64_t total = (int64_t)n * n * (n / 2 + 1);
   const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32);
   { LaunchScope ls_("unpad", st);
-  k_unpad<<<blocks, 256, 0, st>>>(n, P, in, out); }
+  launch(k_unpad, blocks, 256, 0, st, n, P, in, out); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }

@@ -38,6 +38,7 @@ struct Profiler {
 
 extern std::atomic<unsigned long long> g_launches;
 extern thread_local Profiler* t_profiler;
+extern thread_local bool t_overlap;
 
 // Wraps one kernel launch: counts it and, when the calling plan profiles, brackets it with events.
 class LaunchScope {
@@ -70,12 +71,18 @@ class LaunchScope {
 
 // Sets the profiler of the plan used by the current API call.  A call made inside another call
 // that is profiling (an ensemble running its boxes' plans) records into that outer profiler.
+// overlap: whether the call's launches may start before their predecessors end (launch.cuh).
 struct ProfilerGuard {
-  explicit ProfilerGuard(Profiler* p) : prev_(t_profiler) {
+  explicit ProfilerGuard(Profiler* p, bool overlap = false) : prev_(t_profiler), prev_overlap_(t_overlap) {
     if (!(prev_ && prev_->on)) t_profiler = p;
+    t_overlap = overlap;
   }
-  ~ProfilerGuard() { t_profiler = prev_; }
+  ~ProfilerGuard() {
+    t_profiler = prev_;
+    t_overlap = prev_overlap_;
+  }
   Profiler* prev_;
+  bool prev_overlap_;
 };
 
 }  // namespace cola

@@ -26,3 +26,20 @@ def test_fused_deposit_equals_the_integer_deposit(n_p, ng, clumps):
     plan.status()
     for a, b in zip(want, got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n_p,ng,bits", [(48, 64, 16), (48, 128, 12), (64, 96, 16), (96, 256, 16), (96, 256, 20), (48, 64, 8)])
+def test_positions_on_a_mesh_that_is_no_multiple_of_the_lattice(n_p, ng, bits):
+    # the 32-bit lattice offset floor(i ng 2^F / np) against the oracle's, small and box-crossing
+    # displacements (96 on 256: the last size whose bins one block scans)
+    import numpy as np
+
+    import paper_1301_0322_gb300 as cola
+    from oracle import mesh as omesh
+    box = 0.5 * ng
+    plan = cola.Plan(np_side=n_p, ng=ng, box=box, fixed_bits=bits)
+    for sigma in (0.3, 40.0):
+        s = inputs.gaussian_displacements(n_p, sigma, 5)
+        rho, _ = plan.density(torch.from_numpy(s).cuda(), delta=False)
+        got = rho.cpu().numpy().reshape(ng, ng, ng)
+        assert np.array_equal(got, omesh.cic_deposit_fixed(s, n_p, ng, box, bits))
