@@ -27,11 +27,13 @@ __host__ __device__ constexpr int deposit_threads() {
   constexpr int rows = FFTConf<N / 2>::T * TY * TZ, least = N <= 96 ? 256 : (N <= 256 ? 128 : 0);
   return rows < least ? least : rows;
 }
-// resident blocks per SM it is compiled for, by threads per SM; three blocks of 2 x 2 tiles at
-// N = 2048 (64 KB of cell sums each; 80 registers, no spills)
+// resident blocks per SM it is compiled for, by threads per SM (1024: three blocks of 512 threads at
+// 42 registers, 6.9 ms with one -> 5.0; 512: six of 128, 534 -> 509 us; more at 384 or 768 lose);
+// three blocks of 2 x 2 tiles at N = 2048 (64 KB of cell sums each; 80 registers, no spills)
 template <int N, int TY, int TZ>
 __host__ __device__ constexpr int deposit_min_blocks() {
-  constexpr int per_sm = (N <= 96 ? 1024 : (N <= 256 ? 768 : 512)) / deposit_threads<N, TY, TZ>();
+  constexpr int threads = N <= 96 ? 1024 : N <= 256 || N == 512 ? 768 : N == 1024 ? 1536 : 512;
+  constexpr int per_sm = threads / deposit_threads<N, TY, TZ>();
   return N == 2048 && TY * TZ == 4 ? 3 : (per_sm > 0 ? per_sm : 1);
 }
 

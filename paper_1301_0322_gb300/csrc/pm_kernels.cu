@@ -139,14 +139,15 @@ __global__ void __launch_bounds__(256) k_deposit(Geometry g, Tiles tl, const uin
                                                  const int* __restrict__ offsets, int64_t* __restrict__ rho,
                                                  float* __restrict__ delta, float dscale, int* __restrict__ err) {
   pdl_begin();
-  extern __shared__ unsigned long long acc[];
+  extern __shared__ __align__(16) unsigned long long acc[];
   __shared__ int rbeg[9], rpre[10];
   const int ng = g.ng;
   int tyi, tzi;
   tile_of_bin(tl, blockIdx.x, tyi, tzi);
   const int y0 = tyi * TY, z0 = tzi * TZ;
   const int ncell = TZ * TY * ng;
-  for (int i = threadIdx.x; i < ncell; i += blockDim.x) acc[i] = 0ull;
+  for (int i = threadIdx.x; i < ncell / 2; i += blockDim.x)
+    reinterpret_cast<ulonglong2*>(acc)[i] = make_ulonglong2(0ull, 0ull);
   if (threadIdx.x == 0) {
     const int tym = tyi == 0 ? tl.nty - 1 : tyi - 1;
     const int tzm = tzi == 0 ? tl.ntz - 1 : tzi - 1;
@@ -166,25 +167,47 @@ __global__ void __launch_bounds__(256) k_deposit(Geometry g, Tiles tl, const uin
   const int total = rpre[9];
   unsigned* lo = reinterpret_cast<unsigned*>(acc);
   unsigned* hi = lo + ncell;
-  for (int i = threadIdx.x; i < total; i += blockDim.x) {
-    int r = 0;
+  constexpr int U = 4;  // particles in flight per thread
+  for (int base = threadIdx.x; base < total; base += U * blockDim.x) {
+    uint32_t f[U][3];
 #pragma unroll
-    for (int k = 1; k < 9; ++k) r += (i >= rpre[k]) ? 1 : 0;
-    const int64_t pos = rbeg[r] + (i - rpre[r]);
-    const uint4 q = __ldg(rec + pos);
-    const uint32_t f[3] = {q.x, q.y, q.z};
-    acc_cloud<TY, TZ, false>(lo, hi, f, g.fbits, ng, y0, z0);
+    for (int u = 0; u < U; ++u) {
+      const int i = base + u * blockDim.x;
+      if (i < total) {
+        int r = 0;
+#pragma unroll
+        for (int k = 1; k < 9; ++k) r += (i >= rpre[k]) ? 1 : 0;
+        const uint4 q = __ldg(rec + rbeg[r] + (i - rpre[r]));
+        f[u][0] = q.x;
+        f[u][1] = q.y;
+        f[u][2] = q.z;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (base + u * (int)blockDim.x < total) acc_cloud<TY, TZ, false>(lo, hi, f[u], g.fbits, ng, y0, z0);
   }
   __syncthreads();
+  // two cells per thread and access, row by row (no division per cell; ng is a multiple of 4)
   bool overflow = false;
-  for (int i = threadIdx.x; i < ncell; i += blockDim.x) {
-    const int lz = i / (TY * ng), rem = i - lz * (TY * ng);
-    const int ly = rem / ng, x = rem - ly * ng;
-    const int64_t gi = ((int64_t)(z0 + lz) * ng + (y0 + ly)) * ng + x;
-    const unsigned long long v = acc_value(lo, hi, i);
-    overflow |= (v >> 62) != 0ull;
-    if (rho) rho[gi] = (int64_t)v;
-    if (delta) delta[gi] = fmaf(__ull2float_rn(v), dscale, -1.0f);
+  for (int r = 0; r < TY * TZ; ++r) {
+    const int64_t row = ((int64_t)(z0 + r / TY) * ng + (y0 + r % TY)) * ng;
+    const uint2* l2 = reinterpret_cast<const uint2*>(lo + r * ng);
+    const uint2* h2 = reinterpret_cast<const uint2*>(hi + r * ng);
+    for (int x = threadIdx.x; x < ng / 2; x += blockDim.x) {
+      const uint2 l = l2[x], h = h2[x];
+      const unsigned long long a = ((unsigned long long)h.x << 32) | l.x, b = ((unsigned long long)h.y << 32) | l.y;
+      overflow |= ((h.x | h.y) >> 30) != 0u;
+      if (rho) {
+        longlong2 v;
+        v.x = (int64_t)a;
+        v.y = (int64_t)b;
+        reinterpret_cast<longlong2*>(rho + row)[x] = v;
+      }
+      if (delta)
+        reinterpret_cast<float2*>(delta + row)[x] =
+            make_float2(fmaf(__ull2float_rn(a), dscale, -1.0f), fmaf(__ull2float_rn(b), dscale, -1.0f));
+    }
   }
   if (overflow) atomicOr(err, kErrOverflow);
 }
