@@ -71,7 +71,7 @@ typedef struct {
   double a_final;     /* final scale factor (1.0)                                            */
   int32_t deconv;     /* CIC deconvolution power p in 1/W(k)^p of the force: 0, 1 (default), 2 */
   int32_t fixed_bits; /* F: CIC positions are quantised to 2^-F cell (default 16, 8..20)      */
-  int32_t adjoint;    /* 1: also reserve the workspace of cola_step_adjoint (3 more meshes)      */
+  int32_t adjoint;    /* 1: also reserve the workspace of cola_step_adjoint (4 more meshes)      */
   int32_t scheme;     /* Kick/Drift operators, one of COLA_SCHEME_* below (default COLA)         */
   int32_t log_a;      /* 0: steps uniform in a (default, App. A.3.2); 1: uniform in ln a (App. A.2) */
 } cola_config;

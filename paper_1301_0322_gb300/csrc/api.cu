@@ -59,7 +59,7 @@ static size_t layout(cola_plan* p, char* base) {
   w.icC2 = (float2*)take(half_p);
   for (int j = 0; j < 5; ++j) w.icR[j] = (float*)take(sizeof(float) * np3);
   off = std::max(off, pm_end);
-  w.lam_real = p->cfg.adjoint ? (float*)take(sizeof(float) * 3 * ng3) : nullptr;
+  w.lam_real = p->cfg.adjoint ? (float4*)take(sizeof(float4) * ng3) : nullptr;
   return off;
 }
 
@@ -476,12 +476,14 @@ int cola_step_adjoint(cola_plan* plan, int32_t step, const float* s_ckpt, float*
   // term B: deposit lam_v, apply the transposed force operator, gather with the weight gradient
   if ((rc = launch_lambda_deposit(plan->geo, s_ckpt, lam_v, w.lam_real, st))) return rc;
   float2* half[3] = {w.meshA, w.meshG[1], w.meshG[2]};
+  if ((rc = launch_fft_x_r2c3(ng, w.lam_real, half[0], half[1], half[2], plan->Pg, w.tw_g, st))) return rc;
   for (int j = 0; j < 3; ++j)
-    if ((rc = fft3d_r2c(ng, plan->Pg, w.lam_real + j * ng3, half[j], w.tw_g, st))) return rc;
-  if ((rc = launch_kspace_adjoint(ng, plan->Pg, plan->cfg.box, plan->cfg.deconv, half[0], half[1], half[2], st)))
+    if ((rc = launch_fft_cols(ng, false, false, half[j], plan->Pg, w.tw_g, st))) return rc;
+  if ((rc = launch_z_adjoint(ng, plan->Pg, plan->cfg.box, plan->cfg.deconv, half[0], half[1], half[2], w.tw_g, st)))
     return rc;
-  float* phi = w.lam_real;
-  if ((rc = fft3d_c2r(ng, plan->Pg, half[0], phi, w.tw_g, 1.0f, w.err, st))) return rc;
+  float* phi = reinterpret_cast<float*>(w.lam_real);
+  if ((rc = launch_fft_cols(ng, true, false, half[0], plan->Pg, w.tw_g, st))) return rc;
+  if ((rc = launch_fft_x_c2r(ng, half[0], phi, plan->Pg, w.tw_g, 1.0f, false, w.err, st))) return rc;
   const double* row = &plan->coef64[(size_t)step * COLA_NCOEF];
   const double to_cells = (double)ng / plan->cfg.box;
   const double inv_rho_bar = (double)ng3 / (double)plan->geo.np3;

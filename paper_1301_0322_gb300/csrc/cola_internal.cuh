@@ -110,8 +110,8 @@ struct Workspace {
   float2* icC1 = nullptr;
   float2* icC2 = nullptr;
   float* icR[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  // adjoint only: three real meshes for the deposited adjoint (the first doubles as Phi)
-  float* lam_real = nullptr;
+  // adjoint only: a float4 mesh for the deposited adjoint (its start doubles as the real mesh Phi)
+  float4* lam_real = nullptr;
 };
 
 }  // namespace cola
@@ -159,6 +159,11 @@ void twiddle_table(int n, std::vector<float2>& out);
 // ---- launchers (kernels_*.cu) ------------------------------------------------------------
 // FFT passes (fft_kernels.cu)
 int launch_fft_x_r2c(int n, const float* in, float2* out, int64_t nrows, int P, const float2* tw, cudaStream_t st);
+// the first three components of a float4 mesh at once
+int launch_fft_x_r2c3(int n, const float4* in, float2* x, float2* y, float2* z, int P, const float2* tw,
+                      cudaStream_t st);
+int launch_fft_x_c2r(int n, const float2* in, float* out, int P, const float2* tw, float scale, bool sub_sq, int* err,
+                     cudaStream_t st);
 // in place over a half spectrum [n][n][P], along y or along z
 int launch_fft_cols(int n, bool inverse, bool along_z, float2* data, int P, const float2* tw, cudaStream_t st);
 // 3-D helpers built on the passes: r2c (x then y then z) and c2r (z, y, x), layout [n][n][P]
@@ -225,9 +230,11 @@ int launch_ic_assemble(int64_t n3, float d1, float d2, float t1, float t2, const
 // adjoint kernels (adjoint_kernels.cu)
 int launch_adjoint_pre(int64_t n3, int mode, const float* coef, float* lam_s, float* lam_v, float* lam_s1,
                        float* lam_s2, cudaStream_t st);
-int launch_lambda_deposit(const Geometry& g, const float* s, const float* lam, float* out, cudaStream_t st);
-int launch_kspace_adjoint(int ng, int P, double box, int deconv, float2* lx, const float2* ly, const float2* lz,
-                          cudaStream_t st);
+int launch_lambda_deposit(const Geometry& g, const float* s, const float* lam, float4* out, cudaStream_t st);
+// the z pass of the force's transpose (pm_fft_kernels.cu): Phi_k of the three deposited adjoints'
+// spectra after x and y, back along z into lx
+int launch_z_adjoint(int ng, int P, double box, int deconv, float2* lx, const float2* ly, const float2* lz,
+                     const float2* tw, cudaStream_t st);
 int launch_gather_adjoint(const Geometry& g, const float* s, const float* F, const float* phi, const float* lam_v,
                           float* lam_s, float scale_a, float scale_b, int mode, cudaStream_t st);
 int launch_kmul_acc(int n, int P, double box, int kind, int i, int j, float scale, int accumulate, const float2* in,

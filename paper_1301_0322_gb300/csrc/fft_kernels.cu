@@ -70,6 +70,58 @@ __global__ void __launch_bounds__(FFTConf<N / 2>::T * x_rows<N>())
   }
 }
 
+// The same of the first three components of a mesh of float4, into three half spectra: a thread
+// reads its cells once and keeps the components that wait in registers.
+struct Spectra3 {
+  float2* p[3];
+};
+template <int N>
+__global__ void __launch_bounds__(FFTConf<N / 2>::T * x_rows<N>())
+    k_fft_x_r2c3(const float4* __restrict__ in, Spectra3 out, int P, const float2* __restrict__ tw) {
+  using C = FFTConf<N / 2>;
+  constexpr int M = N / 2, T = C::T, E = C::E, RB = x_rows<N>(), LD = xrow_ld<M>();
+  constexpr int R0 = first_radix<C>();
+  extern __shared__ __align__(16) float2 smem[];
+  float2* stab = smem + RB * LD;
+  stw_fill<C, 2>(stab, tw, threadIdx.x, T * RB);
+  const SmemTw<C> stw{stab};
+  const int t = threadIdx.x % T, w = threadIdx.x / T;
+  const int64_t row = (int64_t)blockIdx.x * RB + w;
+  const float4* src = in + row * N;
+  float2* buf = smem + w * LD;
+  auto mem = [&](int n) -> float2& { return buf[xpad<R0>(n)]; };
+  float2 v[3][E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const float4 a = src[2 * (t + T * m)], b = src[2 * (t + T * m) + 1];
+    v[0][m] = make_float2(a.x, b.x);
+    v[1][m] = make_float2(a.y, b.y);
+    v[2][m] = make_float2(a.z, b.z);
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    if constexpr (M == R0) {  // one stage: nothing is exchanged
+      auto load = [&](int n) -> float2 { return v[j][(n - t) / T]; };
+      auto store = [&](int n, float2 x) { mem(n) = x; };
+      fft_1d<M, 2, false>(t, stw, load, mem, store);
+    } else {
+      fft_regs<M, 2, false>(v[j], t, stw, mem);
+      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < E; ++m) mem(t + T * m) = v[j][m];
+    }
+    __syncthreads();
+    float2* dst = out.p[j] + row * P;
+    for (int k = t; k <= M / 2; k += T) {
+      const float2 a = mem(k), b = c_conj(mem(k == 0 ? 0 : M - k));
+      const float2 e = c_scale(c_add(a, b), 0.5f), d = c_scale(c_sub(a, b), 0.5f);
+      const float2 p = c_mul(__ldg(tw + k), make_float2(d.y, -d.x));
+      dst[k] = c_add(e, p);
+      if (2 * k != M) dst[M - k] = c_conj(c_sub(e, p));
+    }
+  }
+}
+
 // Half-spectrum rows -> real rows of length N (unscaled inverse, times `scale`): the persistent
 // inverse-x pass of the force with one component.  SUB_SQ: the rows are not stored but their
 // squares taken off what out holds (the 2LPT source's cross terms).  256^3: 51 us with one item per
@@ -197,6 +249,18 @@ static int x_r2c(const float* in, float2* out, int64_t nrows, int P, const float
   return COLA_OK;
 }
 
+template <int N>
+static int x_r2c3(const float4* in, const Spectra3& out, int P, const float2* tw, cudaStream_t st) {
+  constexpr int M = N / 2, RB = x_rows<N>();
+  constexpr size_t smem = (size_t)(RB * xrow_ld<M>() + stw_size<FFTConf<M>>()) * sizeof(float2);
+  static_assert((N * N) % RB == 0, "whole blocks of rows");
+  allow_smem(k_fft_x_r2c3<N>, smem);
+  LaunchScope ls_(label<N>("r2c"), st);
+  k_fft_x_r2c3<N><<<N * N / RB, FFTConf<M>::T * RB, smem, st>>>(in, out, P, tw);
+  COLA_LAUNCH_CHECK();
+  return COLA_OK;
+}
+
 template <int N, bool SUB_SQ>
 static int x_c2r_t(const float2* in, float* out, int P, const float2* tw, float scale, int* err, cudaStream_t st) {
   constexpr int M = N / 2, RB = c2r3_rows<N>(), NT = FFTConf<M>::T * RB;
@@ -280,6 +344,20 @@ int launch_fft_x_r2c(int n, const float* in, float2* out, int64_t nrows, int P, 
 #define X(N) \
   case N:    \
     return x_r2c<N>(in, out, nrows, P, tw, st);
+    COLA_FOR_SIZES(X)
+#undef X
+    default:
+      return fail(COLA_EUNSUPPORTED, "fft: unsupported length " + std::to_string(n));
+  }
+}
+
+int launch_fft_x_r2c3(int n, const float4* in, float2* x, float2* y, float2* z, int P, const float2* tw,
+                      cudaStream_t st) {
+  const Spectra3 out{{x, y, z}};
+  switch (n) {
+#define X(N) \
+  case N:    \
+    return x_r2c3<N>(in, out, P, tw, st);
     COLA_FOR_SIZES(X)
 #undef X
     default:

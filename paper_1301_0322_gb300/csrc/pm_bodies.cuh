@@ -157,6 +157,25 @@ __device__ __forceinline__ void park_load(const P& park, V (&u)[E]) {
   }
 }
 
+// u += what is parked, 16 words at a time (both at once would not fit in the registers)
+template <class P, int E, class V>
+__device__ __forceinline__ void park_add(const P& park, V (&u)[E]) {
+  constexpr int M = 16 / (2 * lanes_of<V>());  // values in 16 words
+#pragma unroll
+  for (int m0 = 0; m0 < E; m0 += M) {
+    uint32_t r[16];
+    park.load16(m0 / M * 16, r);
+#pragma unroll
+    for (int m = 0; m < M && m0 + m < E; ++m) {
+      if constexpr (lanes_of<V>() == 1)
+        u[m0 + m] = c_add(u[m0 + m], make_float2(__uint_as_float(r[2 * m]), __uint_as_float(r[2 * m + 1])));
+      else
+        u[m0 + m] = c_add(u[m0 + m], V{make_float2(__uint_as_float(r[4 * m]), __uint_as_float(r[4 * m + 1])),
+                                       make_float2(__uint_as_float(r[4 * m + 2]), __uint_as_float(r[4 * m + 3]))});
+    }
+  }
+}
+
 // A thread's place in a group that transforms a strip of W columns, and the group's exchange
 // buffer: columns w K .. of the strip, transform thread t.  Rows of 64 bytes (W = 8) are swapped
 // in pairs according to the parity of n / R0, so that the first stage's stores, which are R0 rows
@@ -485,6 +504,83 @@ __device__ __forceinline__ void z_green_strip(float2* __restrict__ A, float2* __
   if (s.valid) {
 #pragma unroll
     for (int m = 0; m < E; ++m) c_store(a + m * zstep, u[m]);
+  }
+  __syncwarp();
+}
+
+// ---- 3a. the z pass of the force's transpose --------------------------------------------------
+// Phi_k = sum_i conj(i k_i / (k^2 W^p)) Lam_i,k / N^3 of the three deposited adjoints' spectra after
+// their x and y transforms, back along z into lx.  k_x and k_y do not change along z, so k_x Lam_x
+// + k_y Lam_y is one transform; its result is parked while Lam_z is transformed.  One strip
+// (slab = ky) whose copies of lx are under way (next: see cols_strip).
+template <int N, int W, class V, class C, class TW, class P_, class Next>
+__device__ __forceinline__ void z_adjoint_strip(float2* __restrict__ lx, const float2* __restrict__ ly,
+                                                const float2* __restrict__ lz, float kf, int deconv, float norm,
+                                                const TW& stw, const float* sinc2, const StripWalk<N, W, V, C>& s,
+                                                const ColsGroup<N, W, V, C>& mem, const P_& park, Next&& next) {
+  constexpr int K = lanes_of<V>(), E = C::E, T = C::T;
+  constexpr int64_t zstep = (int64_t)T * N * half_pitch<N>();
+  const int t = mem.t, kx = s.kx, ny = signed_mode(s.slab, N);
+  auto k_of = [&](int n) { return n == N / 2 || n == -N / 2 ? 0.0f : kf * (float)n; };
+  V u[E];
+  mem.collect(u, lx + s.first, zstep, s.valid);
+  {
+    const float ky = k_of(ny), kx0 = k_of(kx), kx1 = k_of(kx + K - 1);
+    const float2* p = ly + s.first;
+#pragma unroll
+    for (int m = 0; m < E; ++m, p += zstep) {
+      const V b = s.valid ? c_load<V>(p) : c_zero<V>();
+      if constexpr (K == 1) u[m] = c_fma(ky, b, c_scale(u[m], kx0));
+      else u[m] = c_fma(ky, b, c_scale(u[m], make_float2(kx0, kx1)));
+    }
+  }
+  auto fetch_lz = [&] {
+    mem.sync();
+    mem.fetch(lz + s.first, zstep, s.valid);
+  };
+  fft_regs<N, 1, false, C>(u, t, stw, mem, fetch_lz);
+  park_store(park, u);
+  mem.collect(u, lz + s.first, zstep, s.valid);
+  fft_regs<N, 1, false, C>(u, t, stw, mem);
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const float kz = k_of(signed_mode(t + T * m, N));
+    if constexpr (K == 1) u[m] = c_scale(u[m], kz);
+    else u[m] = c_scale(u[m], make_float2(kz, kz));
+  }
+  __syncwarp();
+  park_add(park, u);
+  {
+    const float kf2 = kf * kf, wy = sinc2[s.slab];
+    const float wxy0 = sinc2[s.valid ? kx : 0] * wy, wxy1 = sinc2[s.valid ? kx + K - 1 : 0] * wy;
+    auto green = [&](int nx, int nz, float wk) {
+      const int m2 = nx * nx + ny * ny + nz * nz;
+      if (m2 == 0) return 0.0f;
+      float den = kf2 * (float)m2;
+      if (deconv) den *= deconv == 2 ? wk * wk : wk;
+      return norm / den;
+    };
+#pragma unroll
+    for (int m = 0; m < E; ++m) {  // -i times the sum
+      const int n = t + T * m, nz = signed_mode(n, N);
+      const float g0 = green(kx, nz, wxy0 * sinc2[n]);
+      if constexpr (K == 1) {
+        u[m] = make_float2(u[m].y * g0, -u[m].x * g0);
+      } else {
+        const float g1 = green(kx + 1, nz, wxy1 * sinc2[n]);
+        u[m] = V{make_float2(u[m].im.x * g0, u[m].im.y * g1), make_float2(-u[m].re.x * g0, -u[m].re.y * g1)};
+      }
+    }
+  }
+  auto after_reads = [&] {
+    mem.sync();
+    next();
+  };
+  fft_regs<N, 1, true, C>(u, t, stw, mem, after_reads);
+  if (s.valid) {
+    float2* p = lx + s.first;
+#pragma unroll
+    for (int m = 0; m < E; ++m) c_store(p + m * zstep, u[m]);
   }
   __syncwarp();
 }

@@ -90,6 +90,16 @@ struct TmemPark {
     }
   }
 
+  // words o .. o + 15 of this thread (o a multiple of 16)
+  __device__ __forceinline__ void load16(int o, uint32_t (&r)[16]) const {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+        "[%16];\n\ttcgen05.wait::ld.sync.aligned;"
+        : COLA_W16(r, 0)
+        : "r"(addr + o)
+        : "memory");
+  }
+
   // gives the columns back (contains a block barrier: every warp's accesses are done)
   __device__ __forceinline__ void close() const {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -114,6 +124,10 @@ struct RegPark {
   __device__ __forceinline__ void load(uint32_t (&r)[N]) const {
 #pragma unroll
     for (int i = 0; i < N; ++i) r[i] = kept[i];
+  }
+  __device__ __forceinline__ void load16(int o, uint32_t (&r)[16]) const {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) r[i] = kept[o + i];
   }
   __device__ __forceinline__ void close() const {}
 };

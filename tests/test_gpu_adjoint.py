@@ -248,3 +248,22 @@ def test_gradient_matches_central_differences_128p_256g(cola):
     # differences scatter by 0.3-5% around its exact adjoint in the same regime at 32^3/64^3
     assert corr > 0.97
     assert np.median(err) < 0.1
+
+
+@pytest.mark.parametrize("n_p,ng,deconv", [(32, 32, 1), (32, 48, 0), (48, 96, 2), (64, 192, 1), (64, 256, 2), (96, 384, 1)])
+def test_force_transpose_at_other_mesh_sizes(cola, n_p, ng, deconv):
+    # the transpose's float4 deposit, x and z passes at one and two columns per thread, every
+    # deconvolution; tolerance of test_step_adjoint_matches_oracle
+    box = 0.8 * ng
+    plan = cola.Plan(np_side=n_p, ng=ng, box=box, deconv=deconv, adjoint=True)
+    row = plan.coeffs()[4]
+    s = inputs.gaussian_displacements(n_p, 1.0, 3)
+    rng = np.random.default_rng(4)
+    lv = rng.standard_normal((3, n_p**3)).astype(np.float32)
+    g_ls, g_lv = torch.zeros((3, n_p**3), device="cuda"), dev(lv)
+    g_l1, g_l2 = torch.zeros_like(g_ls), torch.zeros_like(g_ls)
+    plan.step_adjoint(4, dev(s), g_ls, g_lv, g_l1, g_l2)
+    plan.status()
+    pos = np.mod(omesh.lattice_q(n_p, box) + s.astype(np.float64), box)
+    vjp = row[2] * row[1] * oa.force_vjp(pos, lv.astype(np.float64), n_p**3, ng, box, deconv=deconv)
+    assert np.abs(host(g_ls) - vjp).max() <= 3e-4 * np.abs(vjp).max()
