@@ -41,7 +41,6 @@ static size_t layout(cola_plan* p, char* base) {
   w.rec = (uint4*)take(sizeof(uint4) * np3);
   w.counts = (int*)take(sizeof(int) * p->tiles.nbins);
   w.offsets = (int*)take(sizeof(int) * (p->tiles.nbins + 1));
-  w.cursor = (int*)take(sizeof(int) * p->tiles.nbins);
   w.scan_blocks = (int*)take(sizeof(int) * scan_block_count(p->tiles));
   w.pk_partial = (double*)take(sizeof(double) * power_partial_doubles((int)ng));
   // mesh region: the PM step and the initial conditions reuse the same bytes
@@ -76,14 +75,14 @@ static bool small_mesh(int n) { return n <= 256; }
 
 static int padded_half(int n) { return ((n / 2 + 1) + 3) / 4 * 4; }
 
-// particle binning for positions s: keys -> counts -> offsets -> bin-ordered records
+// particle binning for positions s: ranks and counts -> offsets -> bin-ordered records
 static int bin_particles(cola_plan* p, const float* s, cudaStream_t st) {
   Workspace& w = p->ws;
   int rc = launch_keys(p->geo, p->tiles, s, w.keys, w.counts, w.err, st);
   if (rc) return rc;
-  rc = launch_scan(p->tiles, w.counts, w.offsets, w.cursor, w.scan_blocks, !p->in_ensemble, st);
+  rc = launch_scan(p->tiles, w.counts, w.offsets, w.scan_blocks, !p->in_ensemble, st);
   if (rc) return rc;
-  return launch_scatter(p->geo, s, w.keys, w.cursor, w.rec, st);
+  return launch_scatter(p->geo, p->tiles, s, w.keys, w.offsets, w.rec, st);
 }
 
 // unit force meshes g_j (freal[j]) for positions s

@@ -99,7 +99,7 @@ __host__ __device__ constexpr int ens_tile_ty(int rows, int shape) {
 // ---- persistent kernels -----------------------------------------------------------------------
 // Each kernel walks the items of all boxes: boxes[0 .. nbox), item list starts[0 .. nbox].
 
-// binning, four particles per thread (keys_x4_body, scatter_x4_body)
+// binning, four particles per thread (ranks_x4_body, scatter_x4_body)
 template <int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) ke_keys(const BoxDesc* __restrict__ boxes, const int* __restrict__ starts,
                                               int nbox, const float* __restrict__ s, int* __restrict__ keys,
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) ke_keys(const BoxDesc* __restric
     const int b = cur(starts, item);
     const BoxDesc& d = boxes[b];
     const int64_t q0 = (int64_t)(item - cur.first) * NT * kPartPerThread;
-    keys_x4_body(d.g, d.tl, s + 3 * d.pbase, q0, d.bin_base, keys + d.pbase, counts, d.err);
+    ranks_x4_body(d.g, d.tl, s + 3 * d.pbase, q0, d.bin_base, keys + d.pbase, counts, d.err);
   }
 }
 
@@ -118,14 +118,14 @@ template <int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) ke_scatter(const BoxDesc* __restrict__ boxes,
                                                            const int* __restrict__ starts, int nbox,
                                                            const float* __restrict__ s, const int* __restrict__ keys,
-                                                           int* __restrict__ cursor, uint4* __restrict__ rec) {
+                                                           const int* __restrict__ offsets, uint4* __restrict__ rec) {
   const int total = __ldg(starts + nbox);
   BoxCursor cur(starts, nbox, blockIdx.x);
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
     const int b = cur(starts, item);
     const BoxDesc& d = boxes[b];
     const int64_t q0 = (int64_t)(item - cur.first) * NT * kPartPerThread;
-    scatter_x4_body(d.g, s + 3 * d.pbase, q0, keys + d.pbase, cursor, rec);
+    scatter_x4_body(d.g, d.tl, s + 3 * d.pbase, q0, d.bin_base, keys + d.pbase, offsets, rec);
   }
 }
 
@@ -474,7 +474,6 @@ struct cola_ensemble {
   uint4* rec = nullptr;  // [all particles] bin-ordered records (fixed-point coordinates, lattice index)
   int* counts = nullptr;
   int* offsets = nullptr;
-  int* cursor = nullptr;
   int* scan_blocks = nullptr;
   BoxDesc* d_boxes = nullptr;
   int* d_starts = nullptr;
@@ -686,11 +685,11 @@ int enqueue_binning(cola_ensemble* e, const float* s, cudaStream_t st) {
   COLA_LAUNCH_CHECK();
   Tiles all{};
   all.nbins = e->total_bins;
-  int rc = launch_scan(all, e->counts, e->offsets, e->cursor, e->scan_blocks, false, st);
+  int rc = launch_scan(all, e->counts, e->offsets, e->scan_blocks, false, st);
   if (rc) return rc;
   {
     LaunchScope ls_("ens_scatter", st);
-    ke_scatter<NT><<<e->grid[kKScatter], NT, 0, st>>>(e->d_boxes, sp4, nb, s, e->keys, e->cursor, e->rec);
+    ke_scatter<NT><<<e->grid[kKScatter], NT, 0, st>>>(e->d_boxes, sp4, nb, s, e->keys, e->offsets, e->rec);
   }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
@@ -920,7 +919,6 @@ int cola_ensemble_create(const cola_config* boxes, int32_t nbox, cola_ensemble**
   off += align256(sizeof(uint4) * np_all);                 // bin-ordered records
   off += align256(sizeof(int) * all.nbins);                // counts
   off += align256(sizeof(int) * (all.nbins + 1));          // offsets
-  off += align256(sizeof(int) * all.nbins);                // cursor
   off += align256(sizeof(int) * scan_block_count(all));    // scan block sums
   off += align256(sizeof(BoxDesc) * nbox);                 // box descriptions
   off += align256(sizeof(int) * kENumLists * (nbox + 1));  // work lists
@@ -965,7 +963,6 @@ int cola_ensemble_set_workspace(cola_ensemble* ens, void* dev_ptr, size_t bytes,
   ens->rec = (uint4*)take(sizeof(uint4) * np_all);
   ens->counts = (int*)take(sizeof(int) * all.nbins);
   ens->offsets = (int*)take(sizeof(int) * (all.nbins + 1));
-  ens->cursor = (int*)take(sizeof(int) * all.nbins);
   ens->scan_blocks = (int*)take(sizeof(int) * scan_block_count(all));
   ens->d_boxes = (BoxDesc*)take(sizeof(BoxDesc) * ens->nbox);
   ens->d_starts = (int*)take(sizeof(int) * kENumLists * (ens->nbox + 1));

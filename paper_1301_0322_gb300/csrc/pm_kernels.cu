@@ -13,12 +13,12 @@
 namespace cola {
 
 // ---- binning -------------------------------------------------------------------------------
-// four particles per thread (keys_x4_body)
+// four particles per thread (ranks_x4_body)
 __global__ void __launch_bounds__(256) k_keys_x4(Geometry g, Tiles tl, const float* __restrict__ s,
-                                                 int* __restrict__ keys, int* __restrict__ counts,
+                                                 int* __restrict__ ranks, int* __restrict__ counts,
                                                  int* __restrict__ err) {
   pdl_begin();
-  keys_x4_body(g, tl, s, (int64_t)blockIdx.x * blockDim.x * kPartPerThread, 0, keys, counts, err);
+  ranks_x4_body(g, tl, s, (int64_t)blockIdx.x * blockDim.x * kPartPerThread, 0, ranks, counts, err);
 }
 
 // Exclusive scan of the bin counts in three launches (block sums, scan of the block sums,
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(int nb, int* __restrict__ 
 }
 
 __global__ void __launch_bounds__(1024) k_scan_apply(int n, int* __restrict__ counts, const int* __restrict__ block_sums,
-                                                    int* __restrict__ offsets, int* __restrict__ cursor) {
+                                                    int* __restrict__ offsets) {
   pdl_begin();
   __shared__ int warp_sums[32];
   const int i = blockIdx.x * kScanTile + threadIdx.x;
@@ -82,7 +82,6 @@ __global__ void __launch_bounds__(1024) k_scan_apply(int n, int* __restrict__ co
   const int excl = block_inclusive_scan(x, warp_sums) - x + block_sums[blockIdx.x];
   if (i < n) {
     offsets[i] = excl;
-    cursor[i] = excl;
     counts[i] = 0;
   }
   if (i == n - 1) offsets[n] = excl + x;
@@ -91,8 +90,7 @@ __global__ void __launch_bounds__(1024) k_scan_apply(int n, int* __restrict__ co
 // The three launches as one block for up to kScanOne bins (meshes up to 256): every count is loaded
 // before the first is needed, so the block waits for memory once (6 us in all against 3 x 6).
 constexpr int kScanOne = 32768;
-__global__ void __launch_bounds__(1024) k_scan_one(int n, int* __restrict__ counts, int* __restrict__ offsets,
-                                                   int* __restrict__ cursor) {
+__global__ void __launch_bounds__(1024) k_scan_one(int n, int* __restrict__ counts, int* __restrict__ offsets) {
   pdl_begin();
   constexpr int R = kScanOne / 4096;
   __shared__ int warp_sums[32];
@@ -112,7 +110,6 @@ __global__ void __launch_bounds__(1024) k_scan_one(int n, int* __restrict__ coun
     if (i < n) {
       const int4 o = make_int4(e, e + v[r].x, e + v[r].x + v[r].y, e + v[r].x + v[r].y + v[r].z);
       *reinterpret_cast<int4*>(offsets + i) = o;
-      *reinterpret_cast<int4*>(cursor + i) = o;
       *reinterpret_cast<int4*>(counts + i) = make_int4(0, 0, 0, 0);
     }
     run += total;
@@ -122,11 +119,11 @@ __global__ void __launch_bounds__(1024) k_scan_one(int n, int* __restrict__ coun
 }
 
 // four particles per thread (scatter_x4_body)
-__global__ void __launch_bounds__(256) k_scatter_x4(Geometry g, const float* __restrict__ s,
-                                                    const int* __restrict__ keys, int* __restrict__ cursor,
+__global__ void __launch_bounds__(256) k_scatter_x4(Geometry g, Tiles tl, const float* __restrict__ s,
+                                                    const int* __restrict__ ranks, const int* __restrict__ offsets,
                                                     uint4* __restrict__ rec) {
   pdl_begin();
-  scatter_x4_body(g, s, (int64_t)blockIdx.x * blockDim.x * kPartPerThread, keys, cursor, rec);
+  scatter_x4_body(g, tl, s, (int64_t)blockIdx.x * blockDim.x * kPartPerThread, 0, ranks, offsets, rec);
 }
 
 // ---- deposit ----------------------------------------------------------------------------------
@@ -346,20 +343,19 @@ __global__ void __launch_bounds__(256) k_kick_drift(Geometry g, const float* __r
 // ---- launchers ------------------------------------------------------------------------------------
 static unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
-int launch_keys(const Geometry& g, const Tiles& t, const float* s, int* keys, int* counts, int* err, cudaStream_t st) {
+int launch_keys(const Geometry& g, const Tiles& t, const float* s, int* ranks, int* counts, int* err, cudaStream_t st) {
   { LaunchScope ls_("keys", st);
-  launch(k_keys_x4, blocks_for(g.np3, 256 * kPartPerThread), 256, 0, st, g, t, s, keys, counts, err); }
+  launch(k_keys_x4, blocks_for(g.np3, 256 * kPartPerThread), 256, 0, st, g, t, s, ranks, counts, err); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
 
 int scan_block_count(const Tiles& t) { return (t.nbins + kScanTile - 1) / kScanTile; }
 
-int launch_scan(const Tiles& t, int* counts, int* offsets, int* cursor, int* block_sums, bool one_block,
-                cudaStream_t st) {
+int launch_scan(const Tiles& t, int* counts, int* offsets, int* block_sums, bool one_block, cudaStream_t st) {
   if (one_block && t.nbins <= kScanOne && t.nbins % 4 == 0) {
     LaunchScope ls_("scan_one", st);
-    launch(k_scan_one, 1, 1024, 0, st, t.nbins, counts, offsets, cursor);
+    launch(k_scan_one, 1, 1024, 0, st, t.nbins, counts, offsets);
     COLA_LAUNCH_CHECK();
     return COLA_OK;
   }
@@ -376,16 +372,16 @@ int launch_scan(const Tiles& t, int* counts, int* offsets, int* cursor, int* blo
   COLA_LAUNCH_CHECK();
   {
     LaunchScope ls_("scan_apply", st);
-    launch(k_scan_apply, nb, kScanTile, 0, st, t.nbins, counts, block_sums, offsets, cursor);
+    launch(k_scan_apply, nb, kScanTile, 0, st, t.nbins, counts, block_sums, offsets);
   }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
 
-int launch_scatter(const Geometry& g, const float* s, const int* keys, int* cursor, uint4* rec,
+int launch_scatter(const Geometry& g, const Tiles& t, const float* s, const int* ranks, const int* offsets, uint4* rec,
                    cudaStream_t st) {
   { LaunchScope ls_("scatter", st);
-  launch(k_scatter_x4, blocks_for(g.np3, 256 * kPartPerThread), 256, 0, st, g, s, keys, cursor, rec); }
+  launch(k_scatter_x4, blocks_for(g.np3, 256 * kPartPerThread), 256, 0, st, g, t, s, ranks, offsets, rec); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
