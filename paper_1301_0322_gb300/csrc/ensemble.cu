@@ -186,8 +186,10 @@ __global__ void __launch_bounds__(NT, 512 / NT) ke_cols(const BoxDesc* __restric
   extern __shared__ __align__(16) unsigned long long ens_smem[];
   float2* sm = reinterpret_cast<float2*>(ens_smem);
   __shared__ uint32_t slot;
-  // the longest transforms hold 24 elements a thread
-  const std::conditional_t<KIND == 0, NoPark, Park<NT, 24, float2>> park(&slot);
+  // what is transformed twice stays in registers: one column per thread, at most 24 elements (tensor
+  // memory, shared by the blocks of all sizes, took 3131 us for the z passes and 3549 for the
+  // inverse y passes of the 48 boxes and two more of 64 and 96, registers 1434 and 1853)
+  const std::conditional_t<KIND == 0, NoPark, RegPark<48>> park(&slot);
   const int total = __ldg(starts + nbox);
   BoxCursor cur(starts, nbox, blockIdx.x);
   for (int item = blockIdx.x; item < total; item += gridDim.x) {

@@ -124,8 +124,6 @@ struct ColsCfg {
   using Group = ColsGroup<N, W, V, C>;
 };
 // one thread's E elements, parked (tmem.cuh)
-template <int THREADS, int E, class V>
-using Park = TmemPark<THREADS, (E * lanes_of<V>() * 2 + 15) / 16 * 16>;
 template <class P, int E, class V>
 __device__ __forceinline__ void park_store(const P& park, const V (&u)[E]) {
   uint32_t r[(sizeof(u) / 4 + 15) / 16 * 16] = {};
