@@ -39,18 +39,11 @@ __device__ __forceinline__ V c_load(const float2* p) {
   else return c_interleave(*reinterpret_cast<const float4*>(p));
 }
 template <class V>
-__device__ __forceinline__ V c_load_cg(const float2* p) {
-  if constexpr (lanes_of<V>() == 1) return __ldcg(p);
-  else return c_interleave(__ldcg(reinterpret_cast<const float4*>(p)));
-}
-template <class V>
 __device__ __forceinline__ V c_zero() {
   return V{};
 }
 __device__ __forceinline__ void c_store(float2* p, float2 v) { *p = v; }
 __device__ __forceinline__ void c_store(float2* p, cpair v) { *reinterpret_cast<float4*>(p) = c_deinterleave(v); }
-__device__ __forceinline__ void c_store_cg(float2* p, float2 v) { __stcg(p, v); }
-__device__ __forceinline__ void c_store_cg(float2* p, cpair v) { __stcg(reinterpret_cast<float4*>(p), c_deinterleave(v)); }
 // first-derivative factor i k of both lanes
 __device__ __forceinline__ cpair mul_ik(cpair a, float k) {
   return {p_mul_rn(p_dup(-k), a.im), p_mul_rn(p_dup(k), a.re)};

@@ -162,8 +162,5 @@ __device__ __forceinline__ void acc_cloud(unsigned* lo, unsigned* hi, const uint
     }
   }
 }
-__device__ __forceinline__ unsigned long long acc_value(const unsigned* lo, const unsigned* hi, int i) {
-  return ((unsigned long long)hi[i] << 32) | lo[i];
-}
 
 }  // namespace cola
