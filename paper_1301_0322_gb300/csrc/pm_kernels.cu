@@ -130,8 +130,10 @@ __global__ void __launch_bounds__(256) k_scatter_x4(Geometry g, Tiles tl, const 
 // One block per tile of TY x TZ mesh rows (whole x extent).  It reads the bin-ordered records
 // (fixed-point CIC coordinates, stored by the scatter) of the particles binned to the tile and to
 // the boundary regions of its three lower neighbours, accumulates exact int64 CIC weights in
-// shared memory and writes the rows once (int64 and/or float overdensity).
-template <int TY, int TZ>
+// shared memory and writes the rows once (int64 and/or float overdensity).  The outputs are the
+// caller's: PAIRS stores two cells per access, which takes a rho of 16 and a delta of 8 bytes
+// alignment; other buffers (slices of larger ones) get one cell per access.
+template <int TY, int TZ, bool PAIRS>
 __global__ void __launch_bounds__(256) k_deposit(Geometry g, Tiles tl, const uint4* __restrict__ rec,
                                                  const int* __restrict__ offsets, int64_t* __restrict__ rho,
                                                  float* __restrict__ delta, float dscale, int* __restrict__ err) {
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(256) k_deposit(Geometry g, Tiles tl, const uin
       if (base + u * (int)blockDim.x < total) acc_cloud<TY, TZ, false>(lo, hi, f[u], g.fbits, ng, y0, z0);
   }
   __syncthreads();
-  // two cells per thread and access, row by row (no division per cell; ng is a multiple of 4)
+  // two cells per thread, row by row (no division per cell; ng is a multiple of 4)
   bool overflow = false;
   for (int r = 0; r < TY * TZ; ++r) {
     const int64_t row = ((int64_t)(z0 + r / TY) * ng + (y0 + r % TY)) * ng;
@@ -196,14 +198,25 @@ __global__ void __launch_bounds__(256) k_deposit(Geometry g, Tiles tl, const uin
       const unsigned long long a = ((unsigned long long)h.x << 32) | l.x, b = ((unsigned long long)h.y << 32) | l.y;
       overflow |= ((h.x | h.y) >> 30) != 0u;
       if (rho) {
-        longlong2 v;
-        v.x = (int64_t)a;
-        v.y = (int64_t)b;
-        reinterpret_cast<longlong2*>(rho + row)[x] = v;
+        if constexpr (PAIRS) {
+          longlong2 v;
+          v.x = (int64_t)a;
+          v.y = (int64_t)b;
+          reinterpret_cast<longlong2*>(rho + row)[x] = v;
+        } else {
+          rho[row + 2 * x] = (int64_t)a;
+          rho[row + 2 * x + 1] = (int64_t)b;
+        }
       }
-      if (delta)
-        reinterpret_cast<float2*>(delta + row)[x] =
-            make_float2(fmaf(__ull2float_rn(a), dscale, -1.0f), fmaf(__ull2float_rn(b), dscale, -1.0f));
+      if (delta) {
+        const float2 d = make_float2(fmaf(__ull2float_rn(a), dscale, -1.0f), fmaf(__ull2float_rn(b), dscale, -1.0f));
+        if constexpr (PAIRS) {
+          reinterpret_cast<float2*>(delta + row)[x] = d;
+        } else {
+          delta[row + 2 * x] = d.x;
+          delta[row + 2 * x + 1] = d.y;
+        }
+      }
     }
   }
   if (overflow) atomicOr(err, kErrOverflow);
@@ -386,26 +399,35 @@ int launch_scatter(const Geometry& g, const Tiles& t, const float* s, const int*
   return COLA_OK;
 }
 
-template <int TY, int TZ>
+template <int TY, int TZ, bool PAIRS>
 static int deposit_t(const Geometry& g, const Tiles& t, const uint4* rec, const int* offsets, int64_t* rho,
                      float* delta, int* err, cudaStream_t st) {
   const size_t smem = (size_t)TY * TZ * g.ng * sizeof(unsigned long long);
   if (smem > 227 * 1024) return fail(COLA_EUNSUPPORTED, "deposit tile does not fit in shared memory");
   if (smem > 32 * 1024)
-    COLA_CUDA_CHECK(cudaFuncSetAttribute(k_deposit<TY, TZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    COLA_CUDA_CHECK(cudaFuncSetAttribute(k_deposit<TY, TZ, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const double ng3 = (double)g.ng * g.ng * g.ng;
   const float dscale = (float)(ng3 / ((double)g.np3 * std::ldexp(1.0, 3 * g.fbits)));
   { LaunchScope ls_(TY == 2 ? "deposit_2x2" : (TZ == 2 ? "deposit_4x2" : "deposit_4x4"), st);
-  launch(k_deposit<TY, TZ>, t.nty * t.ntz, 256, smem, st, g, t, rec, offsets, rho, delta, dscale, err); }
+  launch(k_deposit<TY, TZ, PAIRS>, t.nty * t.ntz, 256, smem, st, g, t, rec, offsets, rho, delta, dscale, err); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
 
+template <int TY, int TZ>
+static int deposit_any(const Geometry& g, const Tiles& t, const uint4* rec, const int* offsets, int64_t* rho,
+                       float* delta, int* err, cudaStream_t st) {
+  // (a null output is aligned; rows are multiples of 16 cells)
+  const bool pairs = reinterpret_cast<uintptr_t>(rho) % 16 == 0 && reinterpret_cast<uintptr_t>(delta) % 8 == 0;
+  return pairs ? deposit_t<TY, TZ, true>(g, t, rec, offsets, rho, delta, err, st)
+               : deposit_t<TY, TZ, false>(g, t, rec, offsets, rho, delta, err, st);
+}
+
 int launch_deposit(const Geometry& g, const Tiles& t, const uint4* rec, const int* offsets, int64_t* rho,
                    float* delta, int* err, cudaStream_t st) {
-  if (t.ty == 4 && t.tz == 4) return deposit_t<4, 4>(g, t, rec, offsets, rho, delta, err, st);
-  if (t.ty == 4 && t.tz == 2) return deposit_t<4, 2>(g, t, rec, offsets, rho, delta, err, st);
-  if (t.ty == 2 && t.tz == 2) return deposit_t<2, 2>(g, t, rec, offsets, rho, delta, err, st);
+  if (t.ty == 4 && t.tz == 4) return deposit_any<4, 4>(g, t, rec, offsets, rho, delta, err, st);
+  if (t.ty == 4 && t.tz == 2) return deposit_any<4, 2>(g, t, rec, offsets, rho, delta, err, st);
+  if (t.ty == 2 && t.tz == 2) return deposit_any<2, 2>(g, t, rec, offsets, rho, delta, err, st);
   return fail(COLA_EUNSUPPORTED, "deposit: unsupported tile shape");
 }
 
