@@ -485,7 +485,6 @@ __device__ __forceinline__ void z_green_strip(float2* __restrict__ A, float2* __
 #pragma unroll
     for (int m = 0; m < E; ++m) c_store(gz + m * zstep, u[m]);
   }
-  __syncwarp();
   park_load(park, u);
   auto after_reads = [&] {
     mem.sync();
@@ -539,7 +538,6 @@ __device__ __forceinline__ void z_adjoint_strip(float2* __restrict__ lx, const f
     if constexpr (K == 1) u[m] = c_scale(u[m], kz);
     else u[m] = c_scale(u[m], make_float2(kz, kz));
   }
-  __syncwarp();
   park_add(park, u);
   {
     const float kf2 = kf * kf, wy = sinc2[s.slab];
@@ -603,7 +601,6 @@ __device__ __forceinline__ void y_inv3_strip(float2* __restrict__ B, float2* __r
 #pragma unroll
     for (int m = 0; m < E; ++m) c_store(gy + m * step, u[m]);
   }
-  __syncwarp();
   park_load(park, u);
   auto fetch_gz = [&] {
     mem.sync();

@@ -29,7 +29,9 @@ __host__ __device__ constexpr int tmem_columns(int threads, int words) {
       "=r"(r[o + 12]), "=r"(r[o + 13]), "=r"(r[o + 14]), "=r"(r[o + 15])
 
 // One block's allocation.  The constructor and close() are called by every thread of the block;
-// store and load by whole warps.
+// store and load by whole warps.  Every instruction on tensor memory is .sync.aligned: the lanes of
+// a warp must reach it together, so each function brings them together first, whatever branch the
+// caller took per lane (a column beyond the last one, the mode k = 0) just before.
 template <int THREADS, int WORDS>
 struct TmemPark {
   static constexpr int COLS = tmem_columns(THREADS, WORDS);
@@ -40,6 +42,7 @@ struct TmemPark {
   // (slot: 4 bytes of shared memory; contains a block barrier)
   __device__ __forceinline__ explicit TmemPark(uint32_t* slot) {
     const int warp = threadIdx.x >> 5;
+    __syncwarp();
     if (warp == 0) {
       asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(slot)), "n"(COLS)
                    : "memory");
@@ -56,6 +59,7 @@ struct TmemPark {
   template <int N>
   __device__ __forceinline__ void store(const uint32_t (&r)[N]) const {
     static_assert(N <= WORDS && N % 16 == 0, "whole chunks of this thread's words");
+    __syncwarp();
 #pragma unroll
     for (int o = 0; o < N; o += 16)
       asm volatile(
@@ -69,6 +73,7 @@ struct TmemPark {
   template <int N>
   __device__ __forceinline__ void load(uint32_t (&r)[N]) const {
     static_assert(N <= WORDS && N % 16 == 0, "whole chunks of this thread's words");
+    __syncwarp();
     if constexpr (N % 32 == 0) {
 #pragma unroll
       for (int o = 0; o < N; o += 32)
@@ -92,6 +97,7 @@ struct TmemPark {
 
   // words o .. o + 15 of this thread (o a multiple of 16)
   __device__ __forceinline__ void load16(int o, uint32_t (&r)[16]) const {
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
         "[%16];\n\ttcgen05.wait::ld.sync.aligned;"
