@@ -80,7 +80,7 @@ static int bin_particles(cola_plan* p, const float* s, cudaStream_t st) {
   Workspace& w = p->ws;
   int rc = launch_keys(p->geo, p->tiles, s, w.keys, w.counts, w.err, st);
   if (rc) return rc;
-  rc = launch_scan(p->tiles, w.counts, w.offsets, w.scan_blocks, !p->in_ensemble, st);
+  rc = launch_scan(p->tiles, w.counts, w.offsets, w.scan_blocks, !p->in_ensemble, !bins_ranked(p->geo), st);
   if (rc) return rc;
   return launch_scatter(p->geo, p->tiles, s, w.keys, w.offsets, w.rec, st);
 }

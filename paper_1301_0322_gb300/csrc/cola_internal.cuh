@@ -95,7 +95,7 @@ struct Workspace {
   float2* meshG[3] = {nullptr, nullptr, nullptr};  // [1], [2]: y and z force half spectra ([0] unused)
   float* freal = nullptr;   // 3 x ng^3 force meshes (freal[0..ng^3) doubles as delta)
   // particle binning
-  int* keys = nullptr;  // [np^3]: the particles' ranks in their bins (halo finder: their cells)
+  int* keys = nullptr;  // [np^3]: the particles' ranks in their bins (halo finder: their cells; not ranked: unused)
   // [np^3] in bin order: the particle's fixed-point CIC coordinates f_x, f_y, f_z and its
   // lattice index (one 16-byte record, written and read with one access)
   uint4* rec = nullptr;
@@ -175,11 +175,16 @@ int fft3d_c2r_factor(int n, int P, double box, int kind, int i, int j, float fac
                      float2* tmp, float* out, bool sub_sq, const float2* tw, int* err, cudaStream_t st);
 
 // PM kernels (pm_kernels.cu)
+// whether the binning ranks the particles as it counts them (then ranks holds them), or the scatter
+// takes their places from running cursors (the scan then prepares those)
+bool bins_ranked(const Geometry& g);
 int launch_keys(const Geometry& g, const Tiles& t, const float* s, int* ranks, int* counts, int* err, cudaStream_t st);
 int scan_block_count(const Tiles& t);
-// (one_block: as one launch where the bins are few enough)
-int launch_scan(const Tiles& t, int* counts, int* offsets, int* block_sums, bool one_block, cudaStream_t st);
-int launch_scatter(const Geometry& g, const Tiles& t, const float* s, const int* ranks, const int* offsets, uint4* rec,
+// (one_block: as one launch where the bins are few enough; cursors: !bins_ranked, offsets holds them
+// until the scatter is done)
+int launch_scan(const Tiles& t, int* counts, int* offsets, int* block_sums, bool one_block, bool cursors,
+                cudaStream_t st);
+int launch_scatter(const Geometry& g, const Tiles& t, const float* s, const int* ranks, int* offsets, uint4* rec,
                    cudaStream_t st);
 int launch_deposit(const Geometry& g, const Tiles& t, const uint4* rec, const int* offsets, int64_t* rho,
                    float* delta, int* err, cudaStream_t st);

@@ -687,7 +687,7 @@ int enqueue_binning(cola_ensemble* e, const float* s, cudaStream_t st) {
   COLA_LAUNCH_CHECK();
   Tiles all{};
   all.nbins = e->total_bins;
-  int rc = launch_scan(all, e->counts, e->offsets, e->scan_blocks, false, st);
+  int rc = launch_scan(all, e->counts, e->offsets, e->scan_blocks, false, false, st);
   if (rc) return rc;
   {
     LaunchScope ls_("ens_scatter", st);

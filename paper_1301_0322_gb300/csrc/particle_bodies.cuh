@@ -1,5 +1,5 @@
 // Per-particle device bodies of a COLA force evaluation (Sec. 2 PM code; App. A.3 eq. KDKALC),
-// shared by the single-box kernels and the multi-box (ensemble) kernels.  ranks_x4_body uses
+// shared by the single-box kernels and the multi-box (ensemble) kernels.  The binning bodies use
 // warp-wide votes and must be called by all 32 lanes of a warp; the gather and kick/drift bodies
 // handle the one particle p of the calling thread.
 #pragma once
@@ -59,11 +59,11 @@ __device__ __forceinline__ int64_t x4_first(int64_t q0) {
   return q0 + (int64_t)(threadIdx.x & ~31) * kPartPerThread + (threadIdx.x & 31);
 }
 
-// Rank of each of this thread's particles (see x4_first) among those of its bin (bins from bin_base)
-// and the bin counts: one atomic per distinct bin and round of the warp, whose old value ranks its
-// lanes in lattice order.  The scatter then needs neither the bins' running cursors nor the votes
-// again: it recomputes the bin from the cells of the record (one atomic per bin and round in each
-// of the two kernels before; 512^3 particles: scatter 1273 -> 1020 us, this kernel 935 -> 1015).
+// Binning in two forms (which one a plan takes, with both sides' times: bins_ranked, pm_kernels.cu).
+//
+// Ranked: the count's atomics, one per distinct bin and round of the warp (bins from bin_base), return
+// the rank of its first lane among the particles of the bin, so the scatter takes no atomics: it
+// recomputes the bin from the cells of the record and writes at the bin's offset plus the rank.
 __device__ __forceinline__ void ranks_x4_body(const Geometry& g, const Tiles& tl, const float* __restrict__ s,
                                               int64_t q0, int bin_base, int* __restrict__ ranks,
                                               int* __restrict__ counts, int* __restrict__ err) {
@@ -98,7 +98,7 @@ __device__ __forceinline__ void ranks_x4_body(const Geometry& g, const Tiles& tl
   }
 }
 
-// records of the particles of this thread (see x4_first) into their bins
+// ranked: records of the particles of this thread (see x4_first) into their bins
 __device__ __forceinline__ void scatter_x4_body(const Geometry& g, const Tiles& tl, const float* __restrict__ s,
                                                 int64_t q0, int bin_base, const int* __restrict__ ranks,
                                                 const int* __restrict__ offsets, uint4* __restrict__ rec) {
@@ -128,6 +128,66 @@ __device__ __forceinline__ void scatter_x4_body(const Geometry& g, const Tiles& 
 #pragma unroll
   for (int u = 0; u < U; ++u)
     if (p0 + 32 * u < g.np3) rec[at[u]] = r[u];
+}
+
+// Counted: the count's atomics return nothing, and the scatter takes the places of a warp's lanes from
+// the bin's running cursor, again one atomic per distinct bin and round of the warp.  Nothing per
+// particle is written or read between the two.
+__device__ __forceinline__ void count_x4_body(const Geometry& g, const Tiles& tl, const float* __restrict__ s,
+                                              int64_t q0, int* __restrict__ counts, int* __restrict__ err) {
+  constexpr int U = kPartPerThread;
+  const int64_t p0 = x4_first(q0);
+  const int lane = threadIdx.x & 31;
+  float sx[U], sy[U], sz[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t p = p0 + 32 * u;
+    if (p < g.np3) {
+      sx[u] = __ldg(s + p);
+      sy[u] = __ldg(s + g.np3 + p);
+      sz[u] = __ldg(s + 2 * g.np3 + p);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t p = p0 + 32 * u;
+    const int key = p < g.np3 ? particle_key(g, tl, p, sx[u], sy[u], sz[u], err) : -1;
+    const unsigned peers = __match_any_sync(0xffffffffu, key);
+    if (key >= 0 && lane == __ffs(peers) - 1) atomicAdd(counts + key, __popc(peers));
+  }
+}
+
+__device__ __forceinline__ void place_x4_body(const Geometry& g, const Tiles& tl, const float* __restrict__ s,
+                                              int64_t q0, int* __restrict__ cursors, uint4* __restrict__ rec) {
+  constexpr int U = kPartPerThread;
+  const int64_t p0 = x4_first(q0);
+  const int lane = threadIdx.x & 31;
+  float sx[U], sy[U], sz[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t p = p0 + 32 * u;
+    if (p < g.np3) {
+      sx[u] = __ldg(s + p);
+      sy[u] = __ldg(s + g.np3 + p);
+      sz[u] = __ldg(s + 2 * g.np3 + p);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t p = p0 + 32 * u;
+    int key = -1;
+    uint4 r{};
+    if (p < g.np3) {
+      r = particle_record(g, p, sx[u], sy[u], sz[u]);
+      key = tile_key(tl, (int)(r.y >> g.fbits), (int)(r.z >> g.fbits));
+    }
+    const unsigned peers = __match_any_sync(0xffffffffu, key);
+    const int leader = __ffs(peers) - 1;
+    int base = 0;
+    if (key >= 0 && lane == leader) base = atomicAdd(cursors + key, __popc(peers));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (key >= 0) rec[base + __popc(peers & ((1u << lane) - 1u))] = r;
+  }
 }
 
 // CIC gather of the three force meshes fmesh [3][ng^3] for a cloud that starts at cells c with

@@ -13,12 +13,15 @@
 namespace cola {
 
 // ---- binning -------------------------------------------------------------------------------
-// four particles per thread (ranks_x4_body)
+// four particles per thread (ranks_x4_body or count_x4_body)
+template <bool RANK>
 __global__ void __launch_bounds__(256) k_keys_x4(Geometry g, Tiles tl, const float* __restrict__ s,
                                                  int* __restrict__ ranks, int* __restrict__ counts,
                                                  int* __restrict__ err) {
   pdl_begin();
-  ranks_x4_body(g, tl, s, (int64_t)blockIdx.x * blockDim.x * kPartPerThread, 0, ranks, counts, err);
+  const int64_t q0 = (int64_t)blockIdx.x * blockDim.x * kPartPerThread;
+  if constexpr (RANK) ranks_x4_body(g, tl, s, q0, 0, ranks, counts, err);
+  else count_x4_body(g, tl, s, q0, counts, err);
 }
 
 // Exclusive scan of the bin counts in three launches (block sums, scan of the block sums,
@@ -73,18 +76,21 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(int nb, int* __restrict__ 
   }
 }
 
+// (shift 1: bin i's offset goes to offsets[i + 1], where the scatter takes it as a running cursor and
+// leaves the bin's end, the next one's offset)
 __global__ void __launch_bounds__(1024) k_scan_apply(int n, int* __restrict__ counts, const int* __restrict__ block_sums,
-                                                    int* __restrict__ offsets) {
+                                                    int* __restrict__ offsets, int shift) {
   pdl_begin();
   __shared__ int warp_sums[32];
   const int i = blockIdx.x * kScanTile + threadIdx.x;
   const int x = i < n ? counts[i] : 0;
   const int excl = block_inclusive_scan(x, warp_sums) - x + block_sums[blockIdx.x];
   if (i < n) {
-    offsets[i] = excl;
+    offsets[i + shift] = excl;
     counts[i] = 0;
   }
-  if (i == n - 1) offsets[n] = excl + x;
+  if (shift && i == 0) offsets[0] = 0;
+  if (!shift && i == n - 1) offsets[n] = excl + x;
 }
 
 // The three launches as one block for up to kScanOne bins (meshes up to 256): every count is loaded
@@ -118,12 +124,16 @@ __global__ void __launch_bounds__(1024) k_scan_one(int n, int* __restrict__ coun
   if (threadIdx.x == 0) offsets[n] = run;
 }
 
-// four particles per thread (scatter_x4_body)
+// four particles per thread (scatter_x4_body or place_x4_body, whose cursors are the words from
+// offsets[1], see k_scan_apply)
+template <bool RANK>
 __global__ void __launch_bounds__(256) k_scatter_x4(Geometry g, Tiles tl, const float* __restrict__ s,
-                                                    const int* __restrict__ ranks, const int* __restrict__ offsets,
+                                                    const int* __restrict__ ranks, int* __restrict__ offsets,
                                                     uint4* __restrict__ rec) {
   pdl_begin();
-  scatter_x4_body(g, tl, s, (int64_t)blockIdx.x * blockDim.x * kPartPerThread, 0, ranks, offsets, rec);
+  const int64_t q0 = (int64_t)blockIdx.x * blockDim.x * kPartPerThread;
+  if constexpr (RANK) scatter_x4_body(g, tl, s, q0, 0, ranks, offsets, rec);
+  else place_x4_body(g, tl, s, q0, offsets + 1, rec);
 }
 
 // ---- deposit ----------------------------------------------------------------------------------
@@ -356,17 +366,28 @@ __global__ void __launch_bounds__(256) k_kick_drift(Geometry g, const float* __r
 // ---- launchers ------------------------------------------------------------------------------------
 static unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
+// Ranks pay where the lanes of a warp share bins: meshes no finer than the lattice.  On finer ones, and
+// at the largest lattices, the count waits for more atomics to return than the scatter saves.  us,
+// count + scatter of an evolved state, particles on mesh, ranked / counted: 512^3 on 512^3 1905 /
+// 2012, 768 on 768 6258 / 6394 | 1024 on 1024 14395 / 13928, 256 on 768 314 / 299, 384 on 768 954 /
+// 908, 512 on 1024 2195 / 1996, 768 on 1536 7562 / 6936, 1024 on 2048 20319 / 18184.  At 384 and
+// below they are as good (192 on 384 129 / 128, 128 on 384 45 / 47): ranked, as are the ensembles' bins.
+bool bins_ranked(const Geometry& g) { return g.ng <= 384 || (g.ng <= g.np && g.np <= 768); }
+
 int launch_keys(const Geometry& g, const Tiles& t, const float* s, int* ranks, int* counts, int* err, cudaStream_t st) {
+  const unsigned blocks = blocks_for(g.np3, 256 * kPartPerThread);
   { LaunchScope ls_("keys", st);
-  launch(k_keys_x4, blocks_for(g.np3, 256 * kPartPerThread), 256, 0, st, g, t, s, ranks, counts, err); }
+  if (bins_ranked(g)) launch(k_keys_x4<true>, blocks, 256, 0, st, g, t, s, ranks, counts, err);
+  else launch(k_keys_x4<false>, blocks, 256, 0, st, g, t, s, ranks, counts, err); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
 
 int scan_block_count(const Tiles& t) { return (t.nbins + kScanTile - 1) / kScanTile; }
 
-int launch_scan(const Tiles& t, int* counts, int* offsets, int* block_sums, bool one_block, cudaStream_t st) {
-  if (one_block && t.nbins <= kScanOne && t.nbins % 4 == 0) {
+int launch_scan(const Tiles& t, int* counts, int* offsets, int* block_sums, bool one_block, bool cursors,
+                cudaStream_t st) {
+  if (one_block && !cursors && t.nbins <= kScanOne && t.nbins % 4 == 0) {
     LaunchScope ls_("scan_one", st);
     launch(k_scan_one, 1, 1024, 0, st, t.nbins, counts, offsets);
     COLA_LAUNCH_CHECK();
@@ -385,16 +406,18 @@ int launch_scan(const Tiles& t, int* counts, int* offsets, int* block_sums, bool
   COLA_LAUNCH_CHECK();
   {
     LaunchScope ls_("scan_apply", st);
-    launch(k_scan_apply, nb, kScanTile, 0, st, t.nbins, counts, block_sums, offsets);
+    launch(k_scan_apply, nb, kScanTile, 0, st, t.nbins, counts, block_sums, offsets, cursors ? 1 : 0);
   }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
 
-int launch_scatter(const Geometry& g, const Tiles& t, const float* s, const int* ranks, const int* offsets, uint4* rec,
+int launch_scatter(const Geometry& g, const Tiles& t, const float* s, const int* ranks, int* offsets, uint4* rec,
                    cudaStream_t st) {
+  const unsigned blocks = blocks_for(g.np3, 256 * kPartPerThread);
   { LaunchScope ls_("scatter", st);
-  launch(k_scatter_x4, blocks_for(g.np3, 256 * kPartPerThread), 256, 0, st, g, t, s, ranks, offsets, rec); }
+  if (bins_ranked(g)) launch(k_scatter_x4<true>, blocks, 256, 0, st, g, t, s, ranks, offsets, rec);
+  else launch(k_scatter_x4<false>, blocks, 256, 0, st, g, t, s, ranks, offsets, rec); }
   COLA_LAUNCH_CHECK();
   return COLA_OK;
 }
