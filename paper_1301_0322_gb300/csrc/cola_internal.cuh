@@ -42,6 +42,9 @@ struct Geometry {
   int np_sh1, np_sh2;
   // fixed_axis may take its 32-bit path: 2^22 <= ng 2^F <= 2^30
   int fast32;
+  // ceil(ng 2^(F + 32) / np): floor(i ng 2^F / np) = (i lattice_step) >> 32 for 0 <= i < np, as the
+  // product is above i ng 2^(F + 32) / np by less than i < 2^32 / np
+  uint64_t lattice_step;
 };
 
 // Unsigned 32-bit division by an invariant d >= 1 (Granlund & Montgomery 1994, Sec. 4): with
@@ -55,6 +58,7 @@ inline void set_np_divider(Geometry& g) {
   g.np_sh1 = l < 1 ? l : 1;
   g.np_sh2 = l > 1 ? l - 1 : 0;
   const int64_t period = (int64_t)g.ng << g.fbits;
+  g.lattice_step = (((uint64_t)period << 32) + (uint64_t)g.np - 1) / (uint64_t)g.np;
   g.fast32 = period >= (1LL << 22) && period <= (1LL << 30);
 }
 

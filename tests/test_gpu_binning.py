@@ -44,3 +44,22 @@ def test_both_forms_of_the_binning_bin_the_same_particles():
         plan.status()
         del plan, rho
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("bits", [8, 16, 19, 20])
+@pytest.mark.parametrize("n_p,ng", [(32, 32), (32, 96), (48, 32), (48, 64), (96, 128), (192, 256), (384, 256), (192, 512),
+                                    (384, 512)])
+def test_lattice_offsets(n_p, ng, bits):
+    # undisplaced particles: the density is the product of the axes' lines, which follow from
+    # floor(i ng 2^F / np) alone
+    import paper_1301_0322_gb300 as cola
+    one = 1 << bits
+    f = torch.tensor([i * ng * one // n_p for i in range(n_p)], device="cuda")
+    cell, up = f // one, f % one
+    line = torch.zeros(ng, dtype=torch.int64, device="cuda")
+    line.index_add_(0, cell, one - up)
+    line.index_add_(0, (cell + 1) % ng, up)
+    plan = cola.Plan(np_side=n_p, ng=ng, box=100.0, fixed_bits=bits)
+    rho, _ = plan.density(torch.zeros(3, n_p**3, device="cuda"), delta=False)
+    want = line.view(ng, 1, 1) * line.view(1, ng, 1) * line.view(1, 1, ng)
+    assert torch.equal(rho.view(ng, ng, ng), want)
