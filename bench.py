@@ -159,7 +159,6 @@ def algorithmic_bytes(name, n_p, ng):
         "deposit_4x4": 12 * np3 + 4 * ng3,   # fixed-point coordinates per particle, delta rows written once
         "deposit_4x2": 12 * np3 + 4 * ng3,
         "deposit_2x2": 12 * np3 + 4 * ng3,
-        "kspace_force": 4 * 8 * ng * ng * (ng // 2 + 1),
         "gather_kick_drift": 72 * np3 + 12 * ng3,  # s, v, s1, s2 in, s, v out; 3 force meshes once
         "gather_binned": 28 * np3 + 12 * ng3,  # index + coordinates in, force out; 3 force meshes once
         "gather_binned4": 32 * np3 + 12 * ng3,  # the same with the force as one float4 per particle

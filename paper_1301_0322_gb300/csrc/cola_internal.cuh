@@ -192,8 +192,6 @@ int launch_scatter(const Geometry& g, const Tiles& t, const float* s, const int*
                    cudaStream_t st);
 int launch_deposit(const Geometry& g, const Tiles& t, const uint4* rec, const int* offsets, int64_t* rho,
                    float* delta, int* err, cudaStream_t st);
-int launch_kspace_force(int ng, int P, double box, int deconv, const float2* dk, float2* gx, float2* gy, float2* gz,
-                        cudaStream_t st);
 // the fused mesh passes of one force evaluation (pm_fft_kernels.cu): deposit + x r2c, y pass,
 // z pass with the Green's function, inverse y passes, inverse x passes -> F [3][ng^3]
 // the half spectrum A of the density of the binned particles: the force evaluation's fused

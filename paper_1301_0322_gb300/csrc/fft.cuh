@@ -482,28 +482,20 @@ struct Stockham {
   // Run the stages NS.. of the radix list.  v holds the inputs of the first listed stage.
   // mem(n) -> V& : exchange buffer slot for element n of this thread's sequence.
   // store(n, x)       : final output of element n.
-  // before() / after(): called by every thread just before / after the first block barrier,
-  // the one that separates the first stage's reads of its inputs from the first exchange
-  // writes (a block that reads its inputs from a buffer may hand the buffer on after it).
-  template <int NS, int R, int... Rest, class V, class TW, class Mem, class Store, class Before, class After>
-  __device__ __forceinline__ static void run(V (&v)[E], int t, const TW& tw, Mem& mem, Store& store,
-                                             Before& before, After& after) {
+  template <int NS, int R, int... Rest, class V, class TW, class Mem, class Store>
+  __device__ __forceinline__ static void run(V (&v)[E], int t, const TW& tw, Mem& mem, Store& store) {
     compute<R, NS>(v, t, tw);
     if constexpr (sizeof...(Rest) == 0) {
       static_assert(NS * R == N, "radix list does not multiply to N");
-      if constexpr (NS == 1) before();
       stage_sync(mem);
-      if constexpr (NS == 1) after();
 #pragma unroll
       for (int q = 0; q < E / R; ++q)
 #pragma unroll
         for (int r = 0; r < R; ++r) store(out_index<R, NS>(t, q, r), v[q * R + r]);
     } else {
-      if constexpr (NS == 1) before();
       stage_sync(mem);
-      if constexpr (NS == 1) after();
       exchange<R, NS, FirstRadix<Radices<Rest...>>::value>(v, t, mem);
-      run<NS * R, Rest...>(v, t, tw, mem, store, before, after);
+      run<NS * R, Rest...>(v, t, tw, mem, store);
     }
   }
 
@@ -527,19 +519,16 @@ struct Stockham {
     run_regs<1, Rs...>(v, t, tw, mem, after_reads);
   }
 
-  template <int... Rs, class V, class TW, class Mem, class Store, class Before, class After>
+  template <int... Rs, class V, class TW, class Mem, class Store>
   __device__ __forceinline__ static void run_all(Radices<Rs...>, V (&v)[E], int t, const TW& tw, Mem& mem,
-                                                 Store& store, Before& before, After& after) {
-    run<1, Rs...>(v, t, tw, mem, store, before, after);
+                                                 Store& store) {
+    run<1, Rs...>(v, t, tw, mem, store);
   }
 };
 
-// Convenience wrapper: load the first-stage inputs with load(n) and run the whole transform,
-// with before() / after() around the first block barrier (see Stockham::run).
-template <int N, int TWS, bool INV, class C = FFTConf<N>, class TW, class Load, class Mem, class Store,
-          class Before, class After>
-__device__ __forceinline__ void fft_1d_hooked(int t, const TW& tw, Load& load, Mem& mem, Store& store,
-                                              Before& before, After& after) {
+// Convenience wrapper: load the first-stage inputs with load(n) and run the whole transform.
+template <int N, int TWS, bool INV, class C = FFTConf<N>, class TW, class Load, class Mem, class Store>
+__device__ __forceinline__ void fft_1d(int t, const TW& tw, Load& load, Mem& mem, Store& store) {
   static_assert(C::N == N, "configuration of another length");
   constexpr int E = C::E, T = C::T;
   constexpr int R0 = FirstRadix<typename C::radices>::value;
@@ -548,13 +537,7 @@ __device__ __forceinline__ void fft_1d_hooked(int t, const TW& tw, Load& load, M
   for (int q = 0; q < E / R0; ++q)
 #pragma unroll
     for (int r = 0; r < R0; ++r) v[q * R0 + r] = load(t + T * q + r * (N / R0));
-  Stockham<N, E, TWS, INV>::run_all(typename C::radices{}, v, t, tw, mem, store, before, after);
-}
-
-template <int N, int TWS, bool INV, class C = FFTConf<N>, class TW, class Load, class Mem, class Store>
-__device__ __forceinline__ void fft_1d(int t, const TW& tw, Load& load, Mem& mem, Store& store) {
-  auto none = [] {};
-  fft_1d_hooked<N, TWS, INV, C>(t, tw, load, mem, store, none, none);
+  Stockham<N, E, TWS, INV>::run_all(typename C::radices{}, v, t, tw, mem, store);
 }
 
 // Transform of values in registers: u[m] is element n = t + T m (0 <= m < E) before and after.

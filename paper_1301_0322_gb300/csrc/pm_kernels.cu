@@ -232,50 +232,6 @@ __global__ void __launch_bounds__(256) k_deposit(Geometry g, Tiles tl, const uin
   if (overflow) atomicOr(err, kErrOverflow);
 }
 
-// ---- k-space force --------------------------------------------------------------------------
-__device__ __forceinline__ float sinc_pi(int n, int ng) {
-  if (n == 0) return 1.0f;
-  const float x = (float)n / (float)ng;
-  return sinpif(x) / (3.14159265358979323846f * x);
-}
-
-__global__ void k_kspace_force(int ng, int P, float kf, int deconv, float norm, const float2* __restrict__ dk,
-                               float2* __restrict__ gx, float2* __restrict__ gy, float2* __restrict__ gz) {
-  pdl_begin();
-  const int nh = ng / 2 + 1;
-  const int64_t total = (int64_t)ng * ng * nh;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int kx = (int)(i % nh);
-    const int64_t r = i / nh;
-    const int ky = (int)(r % ng), kz = (int)(r / ng);
-    const int nx = kx, ny = ky < ng / 2 ? ky : ky - ng, nz = kz < ng / 2 ? kz : kz - ng;
-    const int64_t o = r * P + kx;
-    const int m2 = nx * nx + ny * ny + nz * nz;
-    float2 out[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    if (m2 != 0) {
-      float green = norm / (kf * kf * (float)m2);
-      if (deconv) {
-        const float sx = sinc_pi(nx, ng), sy = sinc_pi(ny, ng), sz = sinc_pi(nz, ng);
-        const float w = (sx * sx) * (sy * sy) * (sz * sz);
-        green /= (deconv == 2 ? w * w : w);
-      }
-      const float2 d = dk[o];
-      const float2 val = make_float2(d.x * green, d.y * green);
-      const int half = ng / 2;
-      const float kx_ = (nx == half) ? 0.f : kf * nx;
-      const float ky_ = (ny == -half) ? 0.f : kf * ny;
-      const float kz_ = (nz == -half) ? 0.f : kf * nz;
-      // i k (a + i b) = k (-b + i a)
-      out[0] = make_float2(-kx_ * val.y, kx_ * val.x);
-      out[1] = make_float2(-ky_ * val.y, ky_ * val.x);
-      out[2] = make_float2(-kz_ * val.y, kz_ * val.x);
-    }
-    gx[o] = out[0];
-    gy[o] = out[1];
-    gz[o] = out[2];
-  }
-}
-
 // ---- gather + kick + drift -------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_gather_kick_drift(Geometry g, const float* __restrict__ fmesh,
                                                             float* __restrict__ s, float* __restrict__ v,
@@ -452,18 +408,6 @@ int launch_deposit(const Geometry& g, const Tiles& t, const uint4* rec, const in
   if (t.ty == 4 && t.tz == 2) return deposit_any<4, 2>(g, t, rec, offsets, rho, delta, err, st);
   if (t.ty == 2 && t.tz == 2) return deposit_any<2, 2>(g, t, rec, offsets, rho, delta, err, st);
   return fail(COLA_EUNSUPPORTED, "deposit: unsupported tile shape");
-}
-
-int launch_kspace_force(int ng, int P, double box, int deconv, const float2* dk, float2* gx, float2* gy, float2* gz,
-                        cudaStream_t st) {
-  const float kf = (float)(2.0 * 3.14159265358979323846 / box);
-  const float norm = (float)(1.0 / ((double)ng * ng * ng));
-  const int64_t total = (int64_t)ng * ng * (ng / 2 + 1);
-  const unsigned blocks = (unsigned)std::min<int64_t>(blocks_for(total, 256), 152 * 64);
-  { LaunchScope ls_("kspace_force", st);
-  launch(k_kspace_force, blocks, 256, 0, st, ng, P, kf, deconv, norm, dk, gx, gy, gz); }
-  COLA_LAUNCH_CHECK();
-  return COLA_OK;
 }
 
 int launch_gather_kick_drift(const Geometry& g, const float* fmesh, float* s, float* v, const float* s1,

@@ -38,8 +38,8 @@ __device__ __forceinline__ double widen(float x) {
 // segments' lengths and are kept as integers.  What bounds it is the float64 pipe (two operations
 // per clock and SM): 768^3 modes in 384 shells 1468 us with three float64 adds and as many
 // conversions per segment, 1028 with two adds and none.  Each block then writes its per-shell totals in a
-// fixed order and the finish kernel adds the blocks in block order: the result is
-// deterministic.  NF = 1: one field, partial layout [block][shell][3] = (sum w |k|, sum w P,
+// fixed order and the finish kernel adds the blocks' in a fixed order too (shell_sums: every 32nd
+// block per lane, then the lanes by halves): the result is deterministic.  NF = 1: one field, partial layout [block][shell][3] = (sum w |k|, sum w P,
 // sum w); NF = 2: two fields a, b, [block][shell][5] = (sum w |k|, sum w P_a, sum w P_b,
 // sum w P_ab, sum w) with P_ab from Re(a b^*).  One launch bins the shells b0 .. b1 - 1 of the
 // nbins (the accumulators of a range of shells per warp leave room for more warps than those of
