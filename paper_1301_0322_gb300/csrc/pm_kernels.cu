@@ -332,7 +332,7 @@ bool bins_ranked(const Geometry& g) { return g.ng <= 384 || (g.ng <= g.np && g.n
 
 int launch_keys(const Geometry& g, const Tiles& t, const float* s, int* ranks, int* counts, int* err, cudaStream_t st) {
   const unsigned blocks = blocks_for(g.np3, 256 * kPartPerThread);
-  { LaunchScope ls_("keys", st);
+  { LaunchScope ls_(bins_ranked(g) ? "keys" : "count", st);
   if (bins_ranked(g)) launch(k_keys_x4<true>, blocks, 256, 0, st, g, t, s, ranks, counts, err);
   else launch(k_keys_x4<false>, blocks, 256, 0, st, g, t, s, ranks, counts, err); }
   COLA_LAUNCH_CHECK();
@@ -371,7 +371,7 @@ int launch_scan(const Tiles& t, int* counts, int* offsets, int* block_sums, bool
 int launch_scatter(const Geometry& g, const Tiles& t, const float* s, const int* ranks, int* offsets, uint4* rec,
                    cudaStream_t st) {
   const unsigned blocks = blocks_for(g.np3, 256 * kPartPerThread);
-  { LaunchScope ls_("scatter", st);
+  { LaunchScope ls_(bins_ranked(g) ? "scatter" : "place", st);
   if (bins_ranked(g)) launch(k_scatter_x4<true>, blocks, 256, 0, st, g, t, s, ranks, offsets, rec);
   else launch(k_scatter_x4<false>, blocks, 256, 0, st, g, t, s, ranks, offsets, rec); }
   COLA_LAUNCH_CHECK();
