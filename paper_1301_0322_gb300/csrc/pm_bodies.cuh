@@ -66,7 +66,7 @@ __host__ __device__ constexpr int half_pitch() {
 // into the exchange buffer itself: through the L1 cache each 64-byte row segment held a 128-byte
 // line until it returned, and a kernel that takes 200 KB of shared memory has few lines left.
 // More strips in flight than the shapes below have were slower (768: forward y 659 us with two
-// strips of 8 columns per SM, 747 with three, 1080 with four), as were the E complex pairs of a
+// strips of 8 columns per SM, 716 with three, 1046 with four), as were the E complex pairs of a
 // thread squeezed into fewer registers; wider strips move more of a DRAM page at once (1024: z
 // 4987 us with strips of 8, 4190 with 16).  Event times in us per launch, one column per thread
 // with two-pass or re-read strips -> these shapes (GB300):
@@ -77,6 +77,8 @@ __host__ __device__ constexpr int half_pitch() {
 //    768   734 ->  655      2222 ->  1660             2133 ->  1880
 //   1024  1922 -> 1714      8445 ->  4190             9090 ->  4710
 //   1536  7657 -> 6030     29898 -> 19700            24573 -> 18600
+// (Forward y of the force at 256 is the one that lost; one column per thread on four, five or six
+// blocks per SM takes 25.5, 25 and 29 and no call is faster for it.)
 enum ColsKind { kColsPlain, kColsZ, kColsY };
 template <int N, int W, class V, class C>
 struct ColsGroup;

@@ -102,7 +102,7 @@ __device__ __forceinline__ void acc_add64(unsigned* lo, unsigned* hi, int i, uns
 // cloud's cells are added before the first high word needs a carry, eight atomics in flight per
 // thread instead of one or two.  A block of one or two warps with a clump in its tile is bound by
 // their latency (256^3 mesh, 192^3 clustered particles: 272 -> 248 us); larger blocks hide it and
-// are better off with the fewer registers (512^3 mesh and particles, 2527 us, batched 2741).
+// are better off with the fewer registers (512^3 mesh and particles, 2455 us, batched 2503).
 template <int TY, int TZ, bool BATCH>
 __device__ __forceinline__ void acc_cloud(unsigned* lo, unsigned* hi, const uint32_t (&f)[3], int fbits, int n, int y0,
                                           int z0) {
