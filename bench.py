@@ -18,6 +18,7 @@ collective on the data path ("replicas only", weak scaling); value = sum over ra
 """
 import argparse
 import concurrent.futures
+import glob
 import hashlib
 import json
 import os
@@ -189,16 +190,16 @@ def kernel_source_digest():
 
 
 def measured_traffic(name, workload):
-    """dram read+write bytes per launch from a committed ncu summary, if taken on this source."""
-    path = os.path.join(ROOT, "profiles", "ncu_traffic.json")
-    try:
-        data = json.load(open(path))
-    except Exception:
-        return None
-    rec = data.get(workload, {}).get(name)
-    if not rec or rec.get("source_digest") != kernel_source_digest():
-        return None
-    return rec.get("dram_bytes_per_launch")
+    """dram read+write bytes per launch from a committed ncu summary, if one was taken on this source."""
+    digest = kernel_source_digest()
+    for path in sorted(glob.glob(os.path.join(ROOT, "profiles", "ncu_traffic*.json"))):
+        try:
+            rec = json.load(open(path)).get(workload, {}).get(name)
+        except Exception:
+            continue
+        if rec and rec.get("source_digest") == digest:
+            return rec.get("dram_bytes_per_launch")
+    return None
 
 
 def hbm_peak():
