@@ -174,7 +174,8 @@ int cola_ic_2lpt_adjoint(cola_plan* plan, const float* noise, const float* lam_s
 /* CIC density of the particles at displacements s (Sec. 3.1 analysis; the deposit of the
  * force).  rho_fix (may be NULL): device int64 [ng^3], sum of integer CIC weights with
  * positions quantised to 2^-F cell (sum = np^3 2^3F exactly); delta (may be NULL): device
- * float32 [ng^3], rho_fix ng^3 / (np^3 2^3F) - 1. */
+ * float32 [ng^3], rho_fix ng^3 / (np^3 2^3F) - 1.  Both at any alignment of their elements (a
+ * 16-byte rho_fix and an 8-byte delta are stored two cells at a time). */
 int cola_density(cola_plan* plan, const float* s, int64_t* rho_fix, float* delta, cola_stream stream);
 
 /* Shell-averaged power spectrum of a density mesh (Sec. 3.1): P = (L^3/ng^6) |delta_k|^2 /
